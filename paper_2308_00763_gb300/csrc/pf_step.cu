@@ -858,38 +858,57 @@ __device__ __forceinline__ void fetch_table(const TrackerDev &T, StepSmem<P> &sm
 
 // The strata counts of a thread's elements (phase 1d): C_k of each element from the tile's
 // local prefix loc[m] pinned to the exact boundaries excl / pend, and J = the number of
-// strata points at or below C_k (repeated C values reuse the count: on a peaked posterior
-// most elements repeat the previous C).  nrm is the saved 1/S (the naive study build: S
-// itself).  Force-inlined so that loc and Jr stay in registers.
+// strata points at or below C_k (elements past the tile's last repeat its count).  nrm is
+// the saved 1/S (the naive study build: S itself).  Force-inlined so that loc and Jr stay in
+// registers.
+// The element loop holds no branch (systematic points): the phase is bound by instruction
+// latency, and the eight independent counts overlap.  The tile's last element, whose prefix
+// is the tile's end, and the tracker's last, whose CDF is 1, are set after the loop by the
+// one thread that owns them.
 template <typename A, typename Str>
 __device__ __forceinline__ void strata_counts(const Str &str, const A (&loc)[kItems], int (&Jr)[kItems], A excl,
                                               A pend, A nrm, int eb, int cnt, int k0, int N, A *dbg_cdf,
                                               TrackerState *st) {
     (void)st;
+    if (eb >= cnt) {   // (whole warps, but for one)
+#pragma unroll
+        for (int m = 0; m < kItems; ++m) Jr[m] = N;
+        return;
+    }
 #ifdef PF_NAIVE_RESAMPLE
     const A Sdiv = nrm;
 #else
     const A invS = nrm;
 #endif
+    // the normalised CDF cannot exceed 1; the FP32 scan can round above it
     A cprev = static_cast<A>(-1);
     int jprev = 0;
 #pragma unroll
     for (int m = 0; m < kItems; ++m) {
-        const int e = eb + m;
-        int J = N;                                   // (elements past the tile: unused)
-        if (e < cnt) {
-            const int k = k0 + e;
-            const A Pk = (e == cnt - 1) ? pend : fmin(add_rn(excl, loc[m]), pend);
-            // the normalised CDF cannot exceed 1; the FP32 scan can round above it
-            A C = fmin(PF_NORM(Pk), static_cast<A>(1));
-            if (k == N - 1) { C = static_cast<A>(1); J = N; }
-            else if (C == cprev) J = jprev;          // same CDF value, same count
-            else J = str.count_le(C);
+        const A C = fmin(PF_NORM(fmin(add_rn(excl, loc[m]), pend)), static_cast<A>(1));
+        if constexpr (Str::kReuse) {   // a count costs Philox blocks: repeated values reuse it
+            Jr[m] = C == cprev ? jprev : str.count_le(C);
             cprev = C;
-            jprev = J;
-            if (dbg_cdf) dbg_cdf[PF_IDX(k, N)] = C;
+            jprev = Jr[m];
+        } else {
+            Jr[m] = str.count_le(C);
         }
-        Jr[m] = J;
+    }
+    const int last = cnt - 1 - eb;   // the tile's last element, if this thread owns it
+    if (last < kItems) {
+        const int J = (k0 + cnt == N) ? N : str.count_le(fmin(PF_NORM(pend), static_cast<A>(1)));
+#pragma unroll
+        for (int m = 0; m < kItems; ++m)
+            if (m >= last) Jr[m] = J;
+    }
+    if (dbg_cdf) {
+#pragma unroll
+        for (int m = 0; m < kItems; ++m) {
+            const int e = eb + m;
+            A C = fmin(PF_NORM(e == cnt - 1 ? pend : fmin(add_rn(excl, loc[m]), pend)), static_cast<A>(1));
+            if (k0 + e == N - 1) C = static_cast<A>(1);
+            if (e < cnt) dbg_cdf[PF_IDX(k0 + e, N)] = C;
+        }
     }
 }
 
@@ -1478,28 +1497,31 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
         const acc_t nrm = invS;
 #endif
         int jbl = 0, jprev0 = 0;   // the tile's first count; the count before the thread's first element
+        // The count before a warp's first element: that element's predecessor is the previous
+        // warp's last, whose clamped prefix is the running max of all preceding warps (the
+        // running max at lane 0 of this warp, mex), so the count is taken here from the same
+        // value, with the same arithmetic, as its owner takes it.
+        const acc_t c_beg = fmin(PF_NORM(excl), static_cast<acc_t>(1));
+        const acc_t c_prev = fmin(PF_NORM(fmin(add_rn(excl, mex), pend)), static_cast<acc_t>(1));
+        const auto counts = [&](const auto &str) {
+            strata_counts(str, loc, Jr, excl, pend, nrm, eb, cnt, k0, N, dbg_cdf, st);
+            jbl = (lt == 0) ? 0 : str.count_le(c_beg);
+            if (lane == 0 && tid != 0 && eb < cnt) jprev0 = str.count_le(c_prev);
+            if (tid == 0) jprev0 = jbl;
+        };
         if (T.resampler == kResampleStratified) {
             // (key_lo, key_hi, frame t - 1, tracker id) of the stratum offsets
-            Strata<acc_t, true> str;
-            str.init(N, static_cast<acc_t>(0.5), inv_n, sm.skeys);   // u0 = 1/2 only centres the estimate
-            strata_counts(str, loc, Jr, excl, pend, nrm, eb, cnt, k0, N, dbg_cdf, st);
-            jbl = (lt == 0) ? 0 : str.count_le(fmin(PF_NORM(excl), static_cast<acc_t>(1)));
-            // (see the systematic branch for the count before the thread's first element)
-            if (lane == 0 && tid != 0 && eb < cnt)
-                jprev0 = str.count_le(fmin(PF_NORM(fmin(add_rn(excl, mex), pend)), static_cast<acc_t>(1)));
-            if (tid == 0) jprev0 = jbl;
-        } else {
-            Strata<acc_t, false> str;
+            Stratified<acc_t> str;
+            str.init(N, inv_n, sm.skeys);
+            counts(str);
+        } else if (kF64 || (kMode != kModeStepBig && N <= (1 << 20))) {
+            Systematic<acc_t, true> str;
             str.init(N, u0, inv_n);
-            strata_counts(str, loc, Jr, excl, pend, nrm, eb, cnt, k0, N, dbg_cdf, st);
-            jbl = (lt == 0) ? 0 : str.count_le(fmin(PF_NORM(excl), static_cast<acc_t>(1)));
-            // The count before a warp's first element: that element's predecessor is the
-            // previous warp's last, whose clamped prefix is the running max of all preceding
-            // warps (the running max at lane 0 of this warp, mex), so the count is taken here
-            // from the same value, with the same arithmetic, as its owner takes it.
-            if (lane == 0 && tid != 0 && eb < cnt)
-                jprev0 = str.count_le(fmin(PF_NORM(fmin(add_rn(excl, mex), pend)), static_cast<acc_t>(1)));
-            if (tid == 0) jprev0 = jbl;
+            counts(str);
+        } else if constexpr (!kF64) {
+            Systematic<acc_t, false> str;
+            str.init(N, u0, inv_n);
+            counts(str);
         }
         // Every thread knows the tile's first count and the count before its first element,
         // so the ancestor map's heads go in now (phase 1e fills the gaps): map[jp - jb] =
@@ -1984,7 +2006,7 @@ __global__ void shard_expand_kernel(const A *C, const A *x, const A *y, int64_t 
     const A u0 = sizeof(A) == 8 ? static_cast<A>(uniform_f64(w0)) : static_cast<A>(uniform_f32(w0));
     const A inv_n = sizeof(A) == 8 ? static_cast<A>(1.0 / static_cast<double>(n_global))
                                    : static_cast<A>(1.0f / static_cast<float>(n_global));
-    Strata<A, false> str;
+    Systematic<A, sizeof(A) == 8> str;
     str.init(static_cast<int>(n_global), u0, inv_n);
     const int64_t jb = str.count_le(c_lo);
     for (int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; k < n;
