@@ -170,6 +170,9 @@ struct StepLaunch {
     // own, the shard's prefix starts at shard_lo and its last element is pinned to shard_hi
     // (to 1 on the last shard).  shard = 0 for every other launch.
     int32_t shard = 0, shard_last = 0;
+    // A single tracker (slot 0) whose descriptor and frame reference no kernel on the stream
+    // writes: the launch may read them before the previous one has completed.
+    int32_t preload = 0;
     double shard_lo = 0.0, shard_hi = 0.0, g_M = 0.0, g_invS = 0.0;
 };
 

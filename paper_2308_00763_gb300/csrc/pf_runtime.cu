@@ -416,6 +416,7 @@ static pf_status engine_launch(Engine &e, const uint8_t *override_frame, int64_t
     L.total_tiles = e.total_tiles;
     L.frame_override = override_frame;
     L.pitch_override = override_pitch;
+    L.preload = e.n == 1;
     if (engine_enqueue(e, L, e.stream) != 0) { cudaGetLastError(); return e.fail(PF_ERR_CUDA); }
     e.n_step_launches += 1;
     e.n_kernels += e.kernels_per_step();
@@ -462,6 +463,7 @@ static pf_status engine_run_resident(Engine &e, int32_t count) {
         L.total_tiles = e.total_tiles;
         L.frame_override = nullptr;
         L.pitch_override = 0;
+        L.preload = e.n == 1;
         cudaGraph_t g = nullptr;
         cudaError_t err = cudaStreamBeginCapture(e.capture_stream, cudaStreamCaptureModeThreadLocal);
         int rc = 0;

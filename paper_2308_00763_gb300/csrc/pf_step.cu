@@ -913,9 +913,10 @@ __device__ __forceinline__ void strata_counts(const Str &str, const A (&loc)[kIt
 }
 
 // The descriptor, state and frame reference of launch position ti (slot `slot`) into shared
-// memory, by the whole block (the caller synchronises).
+// memory, by the whole block (the caller synchronises).  what & 1: the descriptor and the
+// frame reference; what & 2: the state.
 template <int P>
-__device__ __forceinline__ void load_descriptor(const StepLaunch &Lp, int slot, int ti, StepSmem<P> &sm) {
+__device__ __forceinline__ void load_descriptor(const StepLaunch &Lp, int slot, int ti, StepSmem<P> &sm, int what) {
     const uint32_t *src_t = reinterpret_cast<const uint32_t *>(Lp.trk + slot);
     const uint32_t *src_s = reinterpret_cast<const uint32_t *>(Lp.states + slot);
     const uint32_t *src_f = reinterpret_cast<const uint32_t *>(Lp.frames + ti);
@@ -923,10 +924,12 @@ __device__ __forceinline__ void load_descriptor(const StepLaunch &Lp, int slot, 
     uint32_t *ds = reinterpret_cast<uint32_t *>(&sm.st);
     uint32_t *df = reinterpret_cast<uint32_t *>(&sm.fr);
     constexpr int nt = sizeof(TrackerDev) / 4, ns = sizeof(TrackerState) / 4, nf = sizeof(FrameRef) / 4;
-    for (int i = threadIdx.x; i < nt + ns + nf; i += kThreads) {
-        if (i < nt) dt[i] = __ldg(src_t + i);
-        else if (i < nt + ns) ds[i - nt] = __ldcg(src_s + i - nt);
-        else df[i - nt - ns] = __ldcg(src_f + i - nt - ns);
+    // state first: one pass of the block loads any of the three sets
+    const int lo = (what & 2) ? 0 : ns, hi = (what & 1) ? ns + nt + nf : ns;
+    for (int i = lo + threadIdx.x; i < hi; i += kThreads) {
+        if (i < ns) ds[i] = __ldcg(src_s + i);
+        else if (i < ns + nt) dt[i - ns] = __ldcg(src_t + i - ns);
+        else df[i - ns - nt] = __ldcg(src_f + i - ns - nt);
     }
 }
 
@@ -971,7 +974,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
     // and kept for the CTA's later tiles of the same tracker (none of them changes
     // before the tracker's last tile of this launch has finished)
     if (ti != sm.cached) {
-        load_descriptor(Lp, slot, ti, sm);
+        load_descriptor(Lp, slot, ti, sm, 3);
         __syncthreads();
         if (tid == 0) sm.cached = ti;
     }
@@ -1835,31 +1838,51 @@ template <int P, int kMode>
 __global__ void __launch_bounds__(kThreads, MinBlocks<P>::value) step_kernel(const StepLaunch Lp) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     StepSmem<P> &sm = *reinterpret_cast<StepSmem<P> *>(smem_raw);
+    // One tracker whose descriptor and frame reference no kernel writes (Lp.preload): they load
+    // while the previous launch drains.
+    if (Lp.ntrk == 1 && Lp.preload) load_descriptor(Lp, 0, 0, sm, 1);
     // Programmatic dependent launch: a launch that follows another step on the same stream
-    // may be scheduled while that one drains; everything it reads (ticket, descriptors,
-    // state, particles) is written by its predecessor, so it first waits for the
-    // predecessor grid to complete, then lets its own successor be scheduled.  (Both are
-    // no-ops for a launch without the programmatic-serialization attribute.)
+    // may be scheduled while that one drains; everything else it reads (ticket, state,
+    // particles) is written by its predecessor, so it waits for the predecessor grid to
+    // complete, then lets its own successor be scheduled.  (Both are no-ops for a launch
+    // without the programmatic-serialization attribute.)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (threadIdx.x == 0) sm.cached = -1;
-    if (Lp.ntrk == 1) {
-        // one tracker: its descriptor and state load while the first ticket is drawn
-        load_descriptor(Lp, Lp.slot_of ? __ldg(&Lp.slot_of[0]) : 0, 0, sm);
-        if (threadIdx.x == 0) sm.cached = 0;
-    }
-    for (;;) {
-        if (threadIdx.x == 0) sm.ticket = atomicAdd(Lp.ticket, 1u);
-        __syncthreads();
-        const uint32_t g = sm.ticket;
-        __syncthreads();
-        if (g >= static_cast<uint32_t>(Lp.total_tiles)) {
-            if (threadIdx.x == 0 && g == static_cast<uint32_t>(Lp.total_tiles) + gridDim.x - 1u)
-                atomicExch(Lp.ticket, 0u);
-            return;
+    if (threadIdx.x == 0) sm.cached = Lp.ntrk == 1 ? 0 : -1;
+    if (Lp.ntrk == 1) load_descriptor(Lp, Lp.slot_of ? __ldg(&Lp.slot_of[0]) : 0, 0, sm, Lp.preload ? 2 : 3);
+    __syncthreads();
+    // Tiles in ticket order.  Where a launch can be a single wave, CTA b's first ticket is b (CTAs
+    // are dispatched in index order, so a tile's predecessors belong to running CTAs) and a
+    // launch of one wave draws none at all: a frame paid a draw before its tile and one to find
+    // none left, about 0.8 us each (with the descriptor load moved before the wait as well, F16
+    // frame at 2^20 particles 23.2 -> 22.1 us, 1000 particles F32 14.9 -> 12.7).  In a longer
+    // launch a ticket is drawn when the CTA is ready for it: drawn a tile ahead, its aggregate
+    // reaches the tiles that look back to it a tile later (2^24 F16 265 -> 329 us).
+    const uint32_t total = static_cast<uint32_t>(Lp.total_tiles);
+    if constexpr (kMode != kModeStepBig) {
+        // every CTA draws once for each tile it ran: total_tiles draws in all
+        for (uint32_t g = blockIdx.x; g < total;) {
+            run_tile<P, kMode>(Lp, static_cast<int>(g), sm);
+            if (total <= gridDim.x) return;
+            __syncthreads();
+            if (threadIdx.x == 0) sm.ticket = gridDim.x + atomicAdd(Lp.ticket, 1u);
+            __syncthreads();
+            g = sm.ticket;
+            if (threadIdx.x == 0 && g == gridDim.x + total - 1u) atomicExch(Lp.ticket, 0u);
         }
-        run_tile<P, kMode>(Lp, static_cast<int>(g), sm);
-        __syncthreads();
+    } else {   // two waves or more (the loop above takes 28 more bytes of spills here, 2.6 % of the frame)
+        for (;;) {
+            if (threadIdx.x == 0) sm.ticket = atomicAdd(Lp.ticket, 1u);
+            __syncthreads();
+            const uint32_t g = sm.ticket;
+            __syncthreads();
+            if (g >= total) {
+                if (threadIdx.x == 0 && g == total + gridDim.x - 1u) atomicExch(Lp.ticket, 0u);
+                return;
+            }
+            run_tile<P, kMode>(Lp, static_cast<int>(g), sm);
+            __syncthreads();
+        }
     }
 }
 
