@@ -27,14 +27,14 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
     return c;
 }
 
-// Uniform on (0,1) from the top 23 bits: ((w >> 9) + 1/2) * 2^-23, exact in FP32 and
-// FP64, so every precision sees the same uniforms.
+// Uniform on (0,1) from the top 23 bits: ((w >> 9) + 1/2) * 2^-23, exact in FP32 and FP64, so
+// every precision sees the same uniforms.  One funnel shift puts the 23 bits under the
+// exponent of [1, 2) and one exact addition takes 1 - 2^-24 off: no integer-to-float
+// conversion (16 a clock per SM against 128), two instructions instead of four.
 __device__ __forceinline__ float uniform_f32(uint32_t w) {
-    return (static_cast<float>(w >> 9) + 0.5f) * 1.1920928955078125e-07f;
+    return __fadd_rn(__uint_as_float(__funnelshift_r(w, 0x7fu, 9)), -0.999999940395355224609375f);
 }
-__device__ __forceinline__ double uniform_f64(uint32_t w) {
-    return (static_cast<double>(w >> 9) + 0.5) * 1.1920928955078125e-07;
-}
+__device__ __forceinline__ double uniform_f64(uint32_t w) { return static_cast<double>(uniform_f32(w)); }
 
 // Box-Muller: two N(0,1) draws from two uniforms.
 __device__ __forceinline__ void box_muller(double ua, double ub, double &nx, double &ny) {

@@ -171,12 +171,6 @@ __device__ uint32_t wait_desc(const LookbackDesc *d, uint64_t tag, TrackerState 
     return 0u;
 }
 
-__device__ __forceinline__ uint32_t atom_add_relaxed(uint32_t *p, uint32_t v) {
-    uint32_t old;
-    asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-    return old;
-}
-
 // Tile partials of the FP32/FP16/BF16 kernels: 32-bit launch tag | float bits per word.
 __device__ __forceinline__ uint64_t partial_tag(uint32_t ep) {   // never 0 (cleared memory)
     return static_cast<uint64_t>(ep % 0x7fffffffu + 1u) << 32;
@@ -273,6 +267,23 @@ __device__ __forceinline__ int pixel_of(float v) {
 }
 __device__ __forceinline__ int pixel_of(double v) {
     return __double2int_rd(fmin(fmax(v, -1048576.0), 1048576.0) + 0.5);
+}
+
+// Column (or row) of a position's pixel in a window: pixel_of(v) - origin as an unsigned value,
+// and a value above any window's extent when the pixel lies outside [-2^20, 2^20] or v is not
+// finite (the caller then takes pixel_of).  floor(v + 1/2) is formed by adding 1.5 * 2^23
+// (FP32; 1.5 * 2^52 in FP64) rounded downwards, which leaves the integer in the low mantissa
+// bits: two additions and an integer subtraction instead of two clamps, an addition and a
+// conversion (a quarter-rate unit).  FP32 for |v| >= 2^22 and any other large or special v:
+// the sum's bits differ from those of 1.5 * 2^23 by at least 2^22 in either direction, which
+// stays outside the window after the subtraction (|origin| < 2^20); FP64: the high word tells.
+__device__ __forceinline__ unsigned window_offset(float v, int origin) {
+    return __float_as_uint(__fadd_rd(__fadd_rn(v, 0.5f), 12582912.0f)) - (0x4B400000u + static_cast<unsigned>(origin));
+}
+__device__ __forceinline__ unsigned window_offset(double v, int origin) {
+    const double t = __dadd_rd(__dadd_rn(v, 0.5), 6755399441055744.0);
+    const bool ok = static_cast<unsigned>(__double2hiint(t)) + 0xBCC80001u <= 1u;
+    return ok ? static_cast<unsigned>(__double2loint(t)) - static_cast<unsigned>(origin) : 0xffffffffu;
 }
 
 // kItems consecutive elements between memory and registers as 16-byte vectors (kItems *
@@ -566,9 +577,9 @@ struct __align__(16) StepSmem {
     using pos_t = typename Tr::pos_t;
     using lik_t = typename Tr::lik_t;
     using acc_t = typename Tr::acc_t;
-    pos_t ax[kTile];          // ancestor positions of the tile (previous frame)
-    pos_t ay[kTile];
-    int32_t J[kTile];         // J[e] = strata assigned to particles k0..k0+e (cumulative)
+    // ancestor positions of the tile (previous frame): x then y, or, in F16 / BF16, one word a
+    // particle (x in the low half), so that the offspring loop gathers both with one load
+    alignas(16) pos_t a[2 * kTile];
     lik_t table[kTableMax];   // likelihood of each pixel of the tile's window
     union {
         uint16_t pre[kRoiMax];      // integer form: row prefix sums of the staged region
@@ -587,7 +598,7 @@ struct __align__(16) StepSmem {
     alignas(16) int warp_incl[kWarps];
     Stats<acc_t> red[kWarps];
     U128 agg_x;               // the tile aggregate (fixed point)
-    int jbeg, jend;
+    int jbeg, jend;           // the tile's offspring are j in [jbeg, jend)
     double u0d;               // resampling offset u0 of the previous frame
     float u0f;
     uint32_t skeys[4];        // stratified resampling: key_lo, key_hi, frame t - 1, tracker id
@@ -600,6 +611,7 @@ struct __align__(16) StepSmem {
     TrackerDev trk;
     TrackerState st;
     FrameRef fr;
+    alignas(16) int32_t J[kTile];   // last: only the step mode allocates it (see counts_array)
 };
 
 // Block-wide merge of per-thread stats, result valid in thread 0.  Each warp takes its
@@ -943,6 +955,22 @@ constexpr int kModeStep = 0, kModeCdf = 1, kModePull = 2;
 // common launch carries none of its code or registers.
 constexpr int kModeStepBig = 3;
 
+// Where a mode keeps J[e], the strata assigned to particles k0 .. k0 + e (cumulative), searched
+// when a tile has more offspring than the map holds.  The step mode stores it always, in its
+// own array: kept in registers until the tile's last count is known, it spills (2^20 F16
+// 21.9 us a frame against 21.6, 65536 20.9 against 20.4).  The tracker-table mode keeps it and
+// stores it over the map when it must (2^24 F16 259 us against 265).  The pull kernel keeps
+// its ancestors' indices there; without the array its CTAs leave 16 KB more to the L1 that its
+// searches run in (2^19 F16 50.8 us against 51.4).
+template <int P, int kMode>
+__device__ __forceinline__ int32_t *counts_array(StepSmem<P> &sm) {
+    return kMode == kModeStep ? sm.J : reinterpret_cast<int32_t *>(sm.map);
+}
+template <int P, int kMode> constexpr size_t smem_bytes() {
+    return kMode == kModeStep ? sizeof(StepSmem<P>) : offsetof(StepSmem<P>, J);
+}
+static_assert(sizeof(uint16_t) * kMapMax == sizeof(int32_t) * kTile, "J fits the map's memory");
+
 // One tile of a launch in mode kMode (trackers of the other modes are skipped).
 template <int P, int kMode>
 __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
@@ -1092,10 +1120,19 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
 #pragma unroll
             for (int m = 0; m < kItems; ++m) { Bits<pos_t>::put(xr, m, xv[m]); Bits<pos_t>::put(yr, m, yv[m]); }
         }
+        if constexpr (Tr::kHalf) {
+            // eight words (x, y) from the four of x and the four of y
+            uint4 *d = reinterpret_cast<uint4 *>(reinterpret_cast<uint32_t *>(sm.a) + eb);
+            d[0] = make_uint4(__byte_perm(xr[0].x, yr[0].x, 0x5410), __byte_perm(xr[0].x, yr[0].x, 0x7632),
+                              __byte_perm(xr[0].y, yr[0].y, 0x5410), __byte_perm(xr[0].y, yr[0].y, 0x7632));
+            d[1] = make_uint4(__byte_perm(xr[0].z, yr[0].z, 0x5410), __byte_perm(xr[0].z, yr[0].z, 0x7632),
+                              __byte_perm(xr[0].w, yr[0].w, 0x5410), __byte_perm(xr[0].w, yr[0].w, 0x7632));
+        } else {
 #pragma unroll
-        for (int k = 0; k < kVp; ++k) {
-            reinterpret_cast<uint4 *>(sm.ax + eb)[k] = xr[k];
-            reinterpret_cast<uint4 *>(sm.ay + eb)[k] = yr[k];
+            for (int k = 0; k < kVp; ++k) {
+                reinterpret_cast<uint4 *>(sm.a + eb)[k] = xr[k];
+                reinterpret_cast<uint4 *>(sm.a + kTile + eb)[k] = yr[k];
+            }
         }
         // clear the ancestor map (its heads are written after the strata are counted)
 #pragma unroll
@@ -1247,9 +1284,9 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             if (e < cnt) {
                 const int a = lo[m] < N ? lo[m] : N - 1;
                 const pos_t xa = Xin[PF_IDX(a, N)], ya = Yin[PF_IDX(a, N)];
-                sm.J[PF_IDX(e, kTile)] = a;
-                sm.ax[PF_IDX(e, kTile)] = xa;
-                sm.ay[PF_IDX(e, kTile)] = ya;
+                counts_array<P, kMode>(sm)[PF_IDX(e, kTile)] = a;
+                sm.a[Tr::kHalf ? 2 * PF_IDX(e, kTile) : PF_IDX(e, kTile)] = xa;
+                sm.a[Tr::kHalf ? 2 * PF_IDX(e, kTile) + 1 : kTile + PF_IDX(e, kTile)] = ya;
                 const float xf = static_cast<float>(to_acc(xa)) + sx, yf = static_cast<float>(to_acc(ya)) + sy;
                 bx0 = fminf(bx0, xf); bx1 = fmaxf(bx1, xf);
                 by0 = fminf(by0, yf); by1 = fmaxf(by1, yf);
@@ -1527,69 +1564,74 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             counts(str);
         }
         // Every thread knows the tile's first count and the count before its first element,
-        // so the ancestor map's heads go in now (phase 1e fills the gaps): map[jp - jb] =
-        // 1 + element, jp the first offspring of each element that has offspring.
+        // so the ancestor map's heads go in now (phase 1e fills the gaps): map[jp - mb] =
+        // 1 + element, jp the first offspring of each element that has offspring, mb the
+        // tile's first offspring rounded down to even (a pair is one aligned word of the map).
         {
-            int jpt = __shfl_up_sync(0xffffffffu, Jr[kItems - 1], 1);
-            if (lane == 0) jpt = jprev0;
+            const int mbl = jbl & ~1;
+            int jp = __shfl_up_sync(0xffffffffu, Jr[kItems - 1], 1);
+            if (lane == 0) jp = jprev0;
+            if (eb < cnt) {
 #pragma unroll
-            for (int m = 0; m < kItems; ++m) {
-                const int jp = m ? Jr[m - 1] : jpt;
-                if (eb + m < cnt && Jr[m] > jp && jp - jbl < kMapMax)
-                    sm.map[PF_IDX(jp - jbl, kMapMax)] = static_cast<uint16_t>(eb + m + 1);
+                for (int m = 0; m < kItems; ++m) {
+                    if (Jr[m] > jp && jp - mbl < kMapMax)
+                        sm.map[PF_IDX(jp - mbl, kMapMax)] = static_cast<uint16_t>(eb + m + 1);
+                    jp = Jr[m];
+                }
+                if constexpr (kMode == kModeStep) store_items(sm.J + eb, Jr);
+                if (eb + kItems >= cnt) sm.jend = Jr[kItems - 1];   // the tile's last element's owner
             }
         }
         if (tid == 0) sm.jbeg = jbl;
-        store_items(sm.J + eb, Jr);
         if (gt) fetch_table<P>(T, sm, wx0, wy0, ww, cells, fv, c1, c2D, den, st);
-        __syncthreads();          // J, jbeg and the likelihood table are complete
+        __syncthreads();          // the heads, jbeg, jend and the likelihood table are complete
         jb = sm.jbeg;
-        je = sm.J[cnt - 1];
+        je = sm.jend;
     } else {
         jb = k0;
         je = k0 + cnt;
         if (gt) fetch_table<P>(T, sm, wx0, wy0, ww, cells, fv, c1, c2D, den, st);
         __syncthreads();          // the likelihood table is complete
     }
-    const int nout = je - jb;
 
     // ------------------------------------------------------------ 1e. ancestor map
-    // map[j - jb] = 1 + tile element that is the ancestor of offspring j: the heads (phase
+    // map[j - mb] = 1 + tile element that is the ancestor of offspring j: the heads (phase
     // 1d; the map was cleared at the start of the tile), then a block-wide running max fills
-    // the gaps.
-    const bool use_map = !kPull && (t > 0) && nout <= kMapMax;
+    // the gaps, two entries of a word at a time.
+    const int mb = jb & ~1;
+    const bool use_map = !kPull && (t > 0) && je - mb <= kMapMax;
     if (use_map) {
         // thread tid fills entries [tid*ch, tid*ch + ch), ch = 8 or 16 (16-byte vectors)
-        const int nv = (nout > kThreads * 8) ? 2 : 1;
+        const int nv = (je - mb > kThreads * 8) ? 2 : 1;
         uint4 *mv = reinterpret_cast<uint4 *>(sm.map) + tid * nv;
         uint4 c0 = mv[0], c1 = make_uint4(0u, 0u, 0u, 0u);
         if (nv == 2) c1 = mv[1];
         uint32_t m2 = __vmaxu2(__vmaxu2(__vmaxu2(c0.x, c0.y), __vmaxu2(c0.z, c0.w)),
                                __vmaxu2(__vmaxu2(c1.x, c1.y), __vmaxu2(c1.z, c1.w)));
         int xm = static_cast<int>(max(m2 & 0xffffu, m2 >> 16));
+        // (a lane without a lane o below gets its own value: no change to a maximum)
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, xm, o);
-            if (lane >= o) xm = max(xm, y);
-        }
+        for (int o = 1; o < 32; o <<= 1) xm = max(xm, __shfl_up_sync(0xffffffffu, xm, o));
         if (lane == 31) sm.warp_imax[warp] = xm;
         int run = __shfl_up_sync(0xffffffffu, xm, 1);
         if (lane == 0) run = 0;
         __syncthreads();
         // the maxima of the preceding warps: lane w < warp holds warp w's (entries are >= 0)
         run = max(run, __reduce_max_sync(0xffffffffu, lane < warp ? sm.warp_imax[lane] : 0));
+        uint32_t r2 = __byte_perm(static_cast<uint32_t>(run), 0u, 0x1010);   // in both halves
         uint32_t w4[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             if (i < 4 * nv) {
-                const int r1 = max(run, static_cast<int>(w4[i] & 0xffffu));
-                const int r2 = max(r1, static_cast<int>(w4[i] >> 16));
-                w4[i] = static_cast<uint32_t>(r1) | (static_cast<uint32_t>(r2) << 16);
-                run = r2;
+                w4[i] = __vmaxu2(__vmaxu2(w4[i], w4[i] << 16), r2);
+                r2 = __byte_perm(w4[i], 0u, 0x3232);
             }
         }
         mv[0] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
         if (nv == 2) mv[1] = make_uint4(w4[4], w4[5], w4[6], w4[7]);
+        __syncthreads();
+    } else if (kMode == kModeStepBig && t > 0) {   // (the barrier above ordered the map's heads)
+        store_items(counts_array<P, kMode>(sm) + eb, Jr);
         __syncthreads();
     }
 
@@ -1621,6 +1663,9 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
     HB2 hbx0 = HalfOps<H>::from_f2(65504.0f, 65504.0f), hbx1 = HalfOps<H>::from_f2(-65504.0f, -65504.0f);
     HB2 hby0 = hbx0, hby1 = hbx1;
 
+    // (What bounds the loop is instruction issue, about 95 a particle.  An aligned map word a pair,
+    // one gathered word an ancestor in F16 / BF16, uniforms by a funnel shift and window_offset
+    // took F32 at 2^20 from 26.1 to 24.0 us a frame, F16 22.1 -> 21.6, REF64 at 200k 262 -> 231.)
     // One pair of offspring (j0, j1) = (2q, 2q + 1).  Compile-time flags: V0 / V1, the
     // particle lies in [jb, je); FAST, frame t > 0 with the ancestor map and no debug
     // arrays (the interior pairs of a tile in production take the FAST copy).
@@ -1630,10 +1675,9 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
         const int j0 = 2 * q, j1 = j0 + 1;
         int e0 = 0, e1 = 0;
         if (kFast) {
-            if (v0) e0 = static_cast<int>(sm.map[PF_IDX(j0 - jb, kMapMax)]) - 1;
-            if (v1) e1 = static_cast<int>(sm.map[PF_IDX(j1 - jb, kMapMax)]) - 1;
-            if (!v0) e0 = e1;
-            if (!v1) e1 = e0;
+            const uint32_t mw = reinterpret_cast<const uint32_t *>(sm.map)[PF_IDX(q - (mb >> 1), kMapMax / 2)];
+            e0 = static_cast<int>(mw & 0xffffu) - 1;
+            e1 = static_cast<int>(mw >> 16) - 1;
         } else if (t > 0) {
             if constexpr (kPull) {
                 // multinomial: the ancestors were gathered into ax/ay at the tile's own
@@ -1641,18 +1685,18 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
                 e0 = j0 - k0;
                 e1 = j1 - k0;
             } else if (use_map) {
-                e0 = v0 ? static_cast<int>(sm.map[PF_IDX(j0 - jb, kMapMax)]) - 1 : 0;
-                e1 = v1 ? static_cast<int>(sm.map[PF_IDX(j1 - jb, kMapMax)]) - 1 : 0;
+                e0 = v0 ? static_cast<int>(sm.map[PF_IDX(j0 - mb, kMapMax)]) - 1 : 0;
+                e1 = v1 ? static_cast<int>(sm.map[PF_IDX(j1 - mb, kMapMax)]) - 1 : 0;
             } else {
-                if (v0) e0 = upper_index(sm.J, cnt, j0);
-                if (v1) e1 = (v0 && sm.J[e0] > j1) ? e0 : upper_index(sm.J, cnt, j1);
+                if (v0) e0 = upper_index(counts_array<P, kMode>(sm), cnt, j0);
+                if (v1) e1 = (v0 && counts_array<P, kMode>(sm)[e0] > j1) ? e0 : upper_index(counts_array<P, kMode>(sm), cnt, j1);
             }
             if (!v0) e0 = e1;
             if (!v1) e1 = e0;
             if (dbg_anc) {
                 if constexpr (kPull) {
-                    if (v0) dbg_anc[PF_IDX(j0, N)] = sm.J[e0];
-                    if (v1) dbg_anc[PF_IDX(j1, N)] = sm.J[e1];
+                    if (v0) dbg_anc[PF_IDX(j0, N)] = counts_array<P, kMode>(sm)[e0];
+                    if (v1) dbg_anc[PF_IDX(j1, N)] = counts_array<P, kMode>(sm)[e1];
                 } else {
                     if (v0) dbg_anc[PF_IDX(j0, N)] = k0 + e0;
                     if (v1) dbg_anc[PF_IDX(j1, N)] = k0 + e1;
@@ -1667,8 +1711,8 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             // ---------------- REF64 / F32: absolute positions, exact-integer likelihood
             acc_t xa0, ya0, xa1, ya1;
             if (t > 0) {
-                xa0 = sm.ax[PF_IDX(e0, kTile)]; ya0 = sm.ay[PF_IDX(e0, kTile)];
-                xa1 = sm.ax[PF_IDX(e1, kTile)]; ya1 = sm.ay[PF_IDX(e1, kTile)];
+                xa0 = sm.a[PF_IDX(e0, kTile)]; ya0 = sm.a[kTile + PF_IDX(e0, kTile)];
+                xa1 = sm.a[PF_IDX(e1, kTile)]; ya1 = sm.a[kTile + PF_IDX(e1, kTile)];
             }
             else {
                 xa0 = xa1 = kF64 ? static_cast<acc_t>(T.init_x) : static_cast<acc_t>(T.init_xf);
@@ -1686,17 +1730,16 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             const acc_t y0 = add_rn(add_rn(ya0, dym), mul_rn(sgy, n0y));
             const acc_t x1 = add_rn(add_rn(xa1, dxm), mul_rn(sgx, n1x));
             const acc_t y1 = add_rn(add_rn(ya1, dym), mul_rn(sgy, n1y));
-            const int px0 = pixel_of(x0), py0 = pixel_of(y0), px1 = pixel_of(x1), py1 = pixel_of(y1);
-            const unsigned cx0 = static_cast<unsigned>(px0 - wx0), cy0 = static_cast<unsigned>(py0 - wy0);
-            const unsigned cx1 = static_cast<unsigned>(px1 - wx0), cy1 = static_cast<unsigned>(py1 - wy0);
+            const unsigned cx0 = window_offset(x0, wx0), cy0 = window_offset(y0, wy0);
+            const unsigned cx1 = window_offset(x1, wx0), cy1 = window_offset(y1, wy0);
             acc_t L0 = static_cast<acc_t>(0), L1 = static_cast<acc_t>(0);
             if (v0) {
                 if (cx0 < static_cast<unsigned>(ww) && cy0 < static_cast<unsigned>(wh)) L0 = sm.table[cy0 * ww + cx0];
-                else L0 = lik_from_sum<acc_t>(disk_sum(fv, sm.w, px0, py0), c1, c2D, den);
+                else L0 = lik_from_sum<acc_t>(disk_sum(fv, sm.w, pixel_of(x0), pixel_of(y0)), c1, c2D, den);
             }
             if (v1) {
                 if (cx1 < static_cast<unsigned>(ww) && cy1 < static_cast<unsigned>(wh)) L1 = sm.table[cy1 * ww + cx1];
-                else L1 = lik_from_sum<acc_t>(disk_sum(fv, sm.w, px1, py1), c1, c2D, den);
+                else L1 = lik_from_sum<acc_t>(disk_sum(fv, sm.w, pixel_of(x1), pixel_of(y1)), c1, c2D, den);
             }
             if (v0 && v1) {
                 if constexpr (sizeof(acc_t) == 8) {
@@ -1724,8 +1767,11 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             using h2 = typename OPS::h2;
             h2 ox, oy;
             if (t > 0) {
-                ox = OPS::pack(sm.ax[PF_IDX(e0, kTile)], sm.ax[PF_IDX(e1, kTile)]);
-                oy = OPS::pack(sm.ay[PF_IDX(e0, kTile)], sm.ay[PF_IDX(e1, kTile)]);
+                const uint32_t a0 = reinterpret_cast<const uint32_t *>(sm.a)[PF_IDX(e0, kTile)];
+                const uint32_t a1 = reinterpret_cast<const uint32_t *>(sm.a)[PF_IDX(e1, kTile)];
+                const uint32_t xw = __byte_perm(a0, a1, 0x5410), yw = __byte_perm(a0, a1, 0x7632);
+                ox = *reinterpret_cast<const h2 *>(&xw);
+                oy = *reinterpret_cast<const h2 *>(&yw);
                 if (shx != 0.0f || shy != 0.0f) {
                     ox = __hadd2(ox, OPS::from_f2(shx, shx));
                     oy = __hadd2(oy, OPS::from_f2(shy, shy));
@@ -1739,16 +1785,14 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             box_muller_fast(uniform_f32(wd.z), uniform_f32(wd.w), c, d);
             ox = __hadd2(ox, OPS::from_f2(dxm + sgx * a, dxm + sgx * c));
             oy = __hadd2(oy, OPS::from_f2(dym + sgy * b, dym + sgy * d));
-            const int px0 = axi + pixel_of(OPS::lo(ox)), py0 = ayi + pixel_of(OPS::lo(oy));
-            const int px1 = axi + pixel_of(OPS::hi(ox)), py1 = ayi + pixel_of(OPS::hi(oy));
-            const unsigned cx0 = static_cast<unsigned>(px0 - wx0), cy0 = static_cast<unsigned>(py0 - wy0);
-            const unsigned cx1 = static_cast<unsigned>(px1 - wx0), cy1 = static_cast<unsigned>(py1 - wy0);
+            const unsigned cx0 = window_offset(OPS::lo(ox), wx0 - axi), cy0 = window_offset(OPS::lo(oy), wy0 - ayi);
+            const unsigned cx1 = window_offset(OPS::hi(ox), wx0 - axi), cy1 = window_offset(OPS::hi(oy), wy0 - ayi);
             const bool in0 = cx0 < static_cast<unsigned>(ww) && cy0 < static_cast<unsigned>(wh);
             const bool in1 = cx1 < static_cast<unsigned>(ww) && cy1 < static_cast<unsigned>(wh);
             H l0 = in0 ? sm.table[cy0 * ww + cx0] : OPS::from_f(0.0f);
             H l1 = in1 ? sm.table[cy1 * ww + cx1] : OPS::from_f(0.0f);
-            if (v0 && !in0) l0 = hk.at(fv, sm.w, px0, py0);
-            if (v1 && !in1) l1 = hk.at(fv, sm.w, px1, py1);
+            if (v0 && !in0) l0 = hk.at(fv, sm.w, axi + pixel_of(OPS::lo(ox)), ayi + pixel_of(OPS::lo(oy)));
+            if (v1 && !in1) l1 = hk.at(fv, sm.w, axi + pixel_of(OPS::hi(ox)), ayi + pixel_of(OPS::hi(oy)));
             if (v0 && v1) {
                 reinterpret_cast<h2 *>(Xout)[PF_IDX(q, N / 2)] = ox;
                 reinterpret_cast<h2 *>(Yout)[q] = oy;
@@ -1976,7 +2020,7 @@ int launch_one(int grid, const StepLaunch &L, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = sizeof(StepSmem<P>);
+    cfg.dynamicSmemBytes = smem_bytes<P, kMode>();
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
