@@ -570,6 +570,69 @@ __device__ __forceinline__ uint32_t warp_disk_sum(const FrameView &f, int px, in
     return __reduce_add_sync(0xffffffffu, s);
 }
 
+// The direct route of the offspring loop: the likelihoods of pixels outside the tile's window,
+// straight from the frame, by all the lanes of `act` that are in the loop's iteration together
+// (miss: which of the lane's two particles need one, 1 and 2).  The lanes take the template's
+// rows of one particle after another, so a particle costs one or two round trips of loads
+// in flight together; its own lane alone read |D| pixels in a nearly serial chain, microseconds
+// that the whole block waited for at the next barrier.  The sums are HalfLik::at's (rows left
+// to right, row sums top to bottom) and disk_sum's, so the bits are.  F16, the paper's motion
+// model at 65536 particles (about four such particles a tile): 20.1 -> 18.6 us a frame.
+template <int P, typename L>
+__device__ __forceinline__ void direct_likelihoods(const TrackerDev &T, const FrameView &f, const int8_t *w, unsigned act,
+                                                   int miss, int px0, int py0, int px1, int py1, L &l0, L &l1) {
+    using acc_t = typename Prec<P>::acc_t;
+    const int lane = threadIdx.x & 31, n = __popc(act), rank = __popc(act & ((1u << lane) - 1u));
+    const int nrow = 2 * f.r + 1;
+    for (unsigned left; (left = __ballot_sync(act, miss != 0)) != 0u;) {
+        const int src = __ffs(static_cast<int>(left)) - 1;
+        const bool first = (miss & 1) != 0;
+        const int px = __shfl_sync(act, first ? px0 : px1, src), py = __shfl_sync(act, first ? py0 : py1, src);
+        L v;
+        if constexpr (Prec<P>::kHalf) {
+            const HalfLik<L> hk = half_lik<L>(T);
+            L hacc = HalfOps<L>::from_f(0.0f);
+            float facc = 0.0f;
+            for (int base = 0; base < nrow; base += n) {
+                const int i = base + rank;
+                L hrow = HalfOps<L>::from_f(0.0f);
+                float frow = 0.0f;
+                if (i < nrow) {
+                    const int hw = w[i];
+#pragma unroll 4
+                    for (int dx = -hw; dx <= hw; ++dx) {
+                        const L tm = hk.term(f.at(px + dx, py + i - f.r));
+                        if (hk.half_acc) hrow = __hadd(hrow, tm); else frow += HalfOps<L>::to_f(tm);
+                    }
+                }
+                unsigned lanes = act;
+                for (int k = base; k < base + n && k < nrow; ++k) {
+                    const int from = __ffs(static_cast<int>(lanes)) - 1;
+                    lanes &= lanes - 1u;
+                    if (hk.half_acc) hacc = __hadd(hacc, __shfl_sync(act, hrow, from));
+                    else facc += __shfl_sync(act, frow, from);
+                }
+            }
+            v = hk.half_acc ? hacc : HalfOps<L>::from_f(facc);
+        } else {
+            constexpr bool kF64 = sizeof(acc_t) == 8;
+            uint32_t s = 0;
+            for (int i = rank; i < nrow; i += n) {
+                const int hw = w[i];
+#pragma unroll 4
+                for (int dx = -hw; dx <= hw; ++dx) s += f.at(px + dx, py + i - f.r);
+            }
+            v = lik_from_sum<acc_t>(__reduce_add_sync(act, s), kF64 ? static_cast<acc_t>(T.c1) : static_cast<acc_t>(T.c1f),
+                                    kF64 ? static_cast<acc_t>(T.c2 * T.D) : static_cast<acc_t>(T.c2Df),
+                                    kF64 ? static_cast<acc_t>(T.den) : static_cast<acc_t>(T.denf));
+        }
+        if (lane == src) {
+            if (first) l0 = v; else l1 = v;
+            miss &= first ? 2 : 0;
+        }
+    }
+}
+
 // Shared memory of the step kernel (dynamic: sizeof(StepSmem<P>) bytes).
 template <int P>
 struct __align__(16) StepSmem {
@@ -1732,14 +1795,18 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             const acc_t y1 = add_rn(add_rn(ya1, dym), mul_rn(sgy, n1y));
             const unsigned cx0 = window_offset(x0, wx0), cy0 = window_offset(y0, wy0);
             const unsigned cx1 = window_offset(x1, wx0), cy1 = window_offset(y1, wy0);
-            acc_t L0 = static_cast<acc_t>(0), L1 = static_cast<acc_t>(0);
-            if (v0) {
-                if (cx0 < static_cast<unsigned>(ww) && cy0 < static_cast<unsigned>(wh)) L0 = sm.table[cy0 * ww + cx0];
-                else L0 = lik_from_sum<acc_t>(disk_sum(fv, sm.w, pixel_of(x0), pixel_of(y0)), c1, c2D, den);
-            }
-            if (v1) {
-                if (cx1 < static_cast<unsigned>(ww) && cy1 < static_cast<unsigned>(wh)) L1 = sm.table[cy1 * ww + cx1];
-                else L1 = lik_from_sum<acc_t>(disk_sum(fv, sm.w, pixel_of(x1), pixel_of(y1)), c1, c2D, den);
+            const bool in0 = cx0 < static_cast<unsigned>(ww) && cy0 < static_cast<unsigned>(wh);
+            const bool in1 = cx1 < static_cast<unsigned>(ww) && cy1 < static_cast<unsigned>(wh);
+            acc_t L0 = v0 && in0 ? sm.table[cy0 * ww + cx0] : static_cast<acc_t>(0);
+            acc_t L1 = v1 && in1 ? sm.table[cy1 * ww + cx1] : static_cast<acc_t>(0);
+            if constexpr (kMode == kModeStepBig) {   // (the tracker's table takes every draw: rarer still)
+                if (v0 && !in0) L0 = lik_from_sum<acc_t>(disk_sum(fv, sm.w, pixel_of(x0), pixel_of(y0)), c1, c2D, den);
+                if (v1 && !in1) L1 = lik_from_sum<acc_t>(disk_sum(fv, sm.w, pixel_of(x1), pixel_of(y1)), c1, c2D, den);
+            } else {
+                const int miss = (v0 && !in0 ? 1 : 0) | (v1 && !in1 ? 2 : 0);
+                const unsigned act = __activemask();
+                if (__any_sync(act, miss != 0))
+                    direct_likelihoods<P>(T, fv, sm.w, act, miss, pixel_of(x0), pixel_of(y0), pixel_of(x1), pixel_of(y1), L0, L1);
             }
             if (v0 && v1) {
                 if constexpr (sizeof(acc_t) == 8) {
@@ -1791,8 +1858,16 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             const bool in1 = cx1 < static_cast<unsigned>(ww) && cy1 < static_cast<unsigned>(wh);
             H l0 = in0 ? sm.table[cy0 * ww + cx0] : OPS::from_f(0.0f);
             H l1 = in1 ? sm.table[cy1 * ww + cx1] : OPS::from_f(0.0f);
-            if (v0 && !in0) l0 = hk.at(fv, sm.w, axi + pixel_of(OPS::lo(ox)), ayi + pixel_of(OPS::lo(oy)));
-            if (v1 && !in1) l1 = hk.at(fv, sm.w, axi + pixel_of(OPS::hi(ox)), ayi + pixel_of(OPS::hi(oy)));
+            if constexpr (kMode == kModeStepBig) {   // (the tracker's table takes every draw: rarer still)
+                if (v0 && !in0) l0 = hk.at(fv, sm.w, axi + pixel_of(OPS::lo(ox)), ayi + pixel_of(OPS::lo(oy)));
+                if (v1 && !in1) l1 = hk.at(fv, sm.w, axi + pixel_of(OPS::hi(ox)), ayi + pixel_of(OPS::hi(oy)));
+            } else {
+                const int miss = (v0 && !in0 ? 1 : 0) | (v1 && !in1 ? 2 : 0);
+                const unsigned act = __activemask();
+                if (__any_sync(act, miss != 0))
+                    direct_likelihoods<P>(T, fv, sm.w, act, miss, axi + pixel_of(OPS::lo(ox)), ayi + pixel_of(OPS::lo(oy)),
+                                          axi + pixel_of(OPS::hi(ox)), ayi + pixel_of(OPS::hi(oy)), l0, l1);
+            }
             if (v0 && v1) {
                 reinterpret_cast<h2 *>(Xout)[PF_IDX(q, N / 2)] = ox;
                 reinterpret_cast<h2 *>(Yout)[q] = oy;
