@@ -108,6 +108,19 @@ inline void fill_tracker_constants(const pf_config &c, TrackerDev &T) {
     T.c1f = static_cast<float>(T.c1);
     T.c2Df = static_cast<float>(T.c2 * T.D);
     T.denf = static_cast<float>(T.den);
+    // template rows and their classes of equal half-width (the half-width falls with |dy|)
+    const int r = c.disk_radius;
+    memset(T.chw, -1, sizeof T.chw);
+    T.ncls = 0;
+    for (int d = 0; d <= r; ++d) {
+        int hw = 0;
+        while ((hw + 1) * (hw + 1) + d * d <= r * r) ++hw;
+        if (d == 0 || hw != T.chw[T.ncls - 1]) T.chw[T.ncls++] = static_cast<int8_t>(hw);
+        T.w[r - d] = T.w[r + d] = static_cast<int8_t>(hw);
+        T.rc[r - d] = T.rc[r + d] = static_cast<uint8_t>(T.ncls - 1);
+    }
+    T.row_terms = 0;
+    for (int k = 0; k < T.ncls; k += 4) T.row_terms += 2 * T.chw[k] + 1;
 }
 
 // The state of a fresh tracker: every particle at the initial position (reading C12).

@@ -130,6 +130,14 @@ struct TrackerDev {
     float init_xf, init_yf, drift_xf, drift_yf, sigma_xf, sigma_yf;
     float c1f, c2Df, denf;
     int32_t window;            // likelihood window: 0 adaptive, 1 always 3.5 sigma, 2 always the full draw range
+    // template rows i = dy + r: half-width (largest w with w^2 + dy^2 <= r^2), and the row's
+    // class: rows of equal half-width share a class, numbered from the widest; chw: half-width
+    // of each class, -1 past the last
+    int8_t w[2 * kMaxRadius + 4];
+    uint8_t rc[2 * kMaxRadius + 4];
+    int8_t chw[kMaxRadius + 8];
+    int32_t ncls;
+    int32_t row_terms;         // terms of the widest class of every four: one pass over a row for all classes
     int64_t j_base;            // global index of particle 0 (a shard of a sharded tracker; even), else 0
     void *px[2], *py[2], *pl[2];
     int32_t *dbg_anc;          // NULL unless PF_FLAG_DEBUG_ARRAYS

@@ -63,6 +63,8 @@ namespace {
 
 constexpr int kWarps = kThreads / 32;
 constexpr int kRoiMax = 2 * kTableMax;     // staged frame pixels (window + template margin)
+// Row sums of the half-form table: words (a half2 of two neighbouring cells, or a float)
+constexpr int kRowWords = 3 * kTile / 2;
 constexpr int kMapMax = 2 * kTile;         // offspring of a tile served by the ancestor map
 constexpr uint32_t kSpinLimit = 1u << 22;  // bounded waits: ~1 s with backoff
 // Half-width of the likelihood window in standard deviations of the transition noise.
@@ -367,16 +369,6 @@ __device__ __forceinline__ void store_items(T *dst, const T (&src)[kItems]) {
 
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
-// Half-width of template row dy (reading C2): the largest w with w^2 + dy^2 <= r^2
-// (|dy| <= r <= 64; the float square root is corrected to the exact integer).
-__device__ __forceinline__ int row_half_width(int r, int dy) {
-    const int q = r * r - dy * dy;
-    int w = static_cast<int>(sqrtf(static_cast<float>(q)));
-    if ((w + 1) * (w + 1) <= q) ++w;
-    if (w * w > q) --w;
-    return w;
-}
-
 struct FrameView {
     const uint8_t *p;
     int64_t pitch;
@@ -387,7 +379,8 @@ struct FrameView {
 };
 
 // Integer sum of the template pixels around (px, py) (the exact form of Eq. 3; reading
-// C4 clamps template pixels to the frame).  w[i] = half-width of template row dy = i - r.
+// C4 clamps template pixels to the frame).  w[i] = half-width of template row dy = i - r
+// (TrackerDev::w).
 __device__ uint32_t disk_sum(const FrameView &f, const int8_t *w, int px, int py) {
     uint32_t s = 0;
     const int r = f.r;
@@ -516,7 +509,7 @@ struct HalfLik {
     }
     // by one warp from the frame: lane l sums rows l, l + 32, ... (each left to right);
     // lane 0 adds the row sums top to bottom.  Valid in lane 0.
-    __device__ H warp_at(const FrameView &f, int px, int py) const {
+    __device__ H warp_at(const FrameView &f, const int8_t *w, int px, int py) const {
         const int lane = threadIdx.x & 31, nrow = 2 * f.r + 1;
         H hacc = HalfOps<H>::from_f(0.0f);
         float facc = 0.0f;
@@ -526,7 +519,7 @@ struct HalfLik {
             float frow = 0.0f;
             if (i < nrow) {
                 const int dy = i - f.r;
-                const int hw = row_half_width(f.r, dy);
+                const int hw = w[i];
                 for (int dx = -hw; dx <= hw; ++dx) {
                     const H tm = term(f.at(px + dx, py + dy));
                     if (half_acc) hrow = __hadd(hrow, tm); else frow += HalfOps<H>::to_f(tm);
@@ -560,11 +553,11 @@ __device__ __forceinline__ HalfLik<H> half_lik(const TrackerDev &T) {
 }
 
 // Integer disk sum by one warp (lanes take template rows; exact, so the order is free).
-__device__ __forceinline__ uint32_t warp_disk_sum(const FrameView &f, int px, int py) {
+__device__ __forceinline__ uint32_t warp_disk_sum(const FrameView &f, const int8_t *w, int px, int py) {
     const int lane = threadIdx.x & 31, nrow = 2 * f.r + 1;
     uint32_t s = 0;
     for (int i = lane; i < nrow; i += 32) {
-        const int hw = row_half_width(f.r, i - f.r);
+        const int hw = w[i];
         for (int dx = -hw; dx <= hw; ++dx) s += f.at(px + dx, py + i - f.r);
     }
     return __reduce_add_sync(0xffffffffu, s);
@@ -667,14 +660,15 @@ struct __align__(16) StepSmem {
     uint32_t skeys[4];        // stratified resampling: key_lo, key_hi, frame t - 1, tracker id
     int win_x0, win_y0, win_w, win_h;   // likelihood table window (win_w = 0: none)
     int qmin;
-    int8_t w[2 * kMaxRadius + 1];
     uint32_t ticket;
     uint32_t last;
     int cached;               // tracker whose descriptor / state / frame are loaded below
     TrackerDev trk;
     TrackerState st;
     FrameRef fr;
-    alignas(16) int32_t J[kTile];   // last: only the step mode allocates it (see counts_array)
+    // last: only the step mode allocates them (see counts_array and row_words)
+    alignas(16) uint32_t rows[Tr::kHalf ? kRowWords : 4];   // half form: row sums of the table's rows
+    alignas(16) int32_t J[kTile];
 };
 
 // Block-wide merge of per-thread stats, result valid in thread 0.  Each warp takes its
@@ -919,13 +913,13 @@ __device__ __forceinline__ void fetch_table(const TrackerDev &T, StepSmem<P> &sm
             if (built) {
                 payload = static_cast<uint32_t>(v);
             } else {
-                const H h = half_lik<H>(T).at(fv, sm.w, gx0 + c % gw, gy0 + c / gw);
+                const H h = half_lik<H>(T).at(fv, sm.trk.w, gx0 + c % gw, gy0 + c / gw);
                 payload = static_cast<uint32_t>(*reinterpret_cast<const unsigned short *>(&h));
             }
             const unsigned short bits = static_cast<unsigned short>(payload);
             sm.table[PF_IDX(c, kTableMax)] = *reinterpret_cast<const H *>(&bits);
         } else {
-            payload = built ? static_cast<uint32_t>(v) : disk_sum(fv, sm.w, gx0 + c % gw, gy0 + c / gw);
+            payload = built ? static_cast<uint32_t>(v) : disk_sum(fv, sm.trk.w, gx0 + c % gw, gy0 + c / gw);
             sm.table[PF_IDX(c, kTableMax)] = lik_from_sum<A>(payload, c1, c2D, den);
         }
     }
@@ -1029,10 +1023,88 @@ template <int P, int kMode>
 __device__ __forceinline__ int32_t *counts_array(StepSmem<P> &sm) {
     return kMode == kModeStep ? sm.J : reinterpret_cast<int32_t *>(sm.map);
 }
+// The words of the table's row sums: their own array in the step mode, in the pull mode the map,
+// which has no use there but for the ancestors' indices when debug arrays are on (24 KB less shared memory, which the L1 keeps for its searches and gathers).
+template <int P, int kMode>
+__device__ __forceinline__ uint32_t *row_words(StepSmem<P> &sm) {
+    return kMode == kModeStep ? sm.rows : reinterpret_cast<uint32_t *>(sm.map);
+}
 template <int P, int kMode> constexpr size_t smem_bytes() {
-    return kMode == kModeStep ? sizeof(StepSmem<P>) : offsetof(StepSmem<P>, J);
+    return kMode == kModeStep ? sizeof(StepSmem<P>) : offsetof(StepSmem<P>, rows);
 }
 static_assert(sizeof(uint16_t) * kMapMax == sizeof(int32_t) * kTile, "J fits the map's memory");
+
+// The half-form table of a window from the staged terms, by row sums.  A cell is the sum of its
+// template rows top to bottom, each summed left to right (HalfLik); a row's sum depends only on
+// its half-width, its place and its frame row, so rows of equal half-width (a class) are the
+// same sum for every cell that has the row at some dy.  Phase A sums every (class, frame row,
+// cell column) once, four classes at a time from one pass over the row's terms; phase B adds
+// each cell's 2 r + 1 row sums.  Every cell performs the additions of HalfLik::from_terms in the
+// same order (kPair: two neighbouring cells in the lanes of a half2, accumulated in half; else
+// one cell a word, accumulated in FP32).  A disk of radius 5 has 4 classes for 11 rows (28
+// additions instead of 81 a cell and row phase), radius 10 has 7 for 21 (95 instead of 317),
+// and the row sums spread over every thread of the block where one thread a cell left most
+// idle in a chain of |D| dependent additions.  Windows whose row sums do not fit are done in
+// bands of `band` cell rows.  Measured us a
+// frame, cells one by one -> row sums: BF16 300007 particles r = 10 20.9 -> 19.0, F16 4096
+// particles r = 12 18.8 -> 16.1; F16 2^20 particles r = 5 21.8 -> 22.0 (there the tiles build
+// their tables while they wait for their predecessors).
+template <int P, int kMode, bool kPair>
+__device__ __forceinline__ void table_by_rows(StepSmem<P> &sm, int rw, int pw, int ww, int wh, int band,
+                                              TrackerState *st) {
+    (void)st;
+    using H = typename Prec<P>::pos_t;
+    using R = typename std::conditional<kPair, __half2, float>::type;
+    const TrackerDev &T = sm.trk;
+    const int r = T.r, ncls = T.ncls, tid = threadIdx.x;
+    R *rows = reinterpret_cast<R *>(row_words<P, kMode>(sm));
+    const auto zero = [] { if constexpr (kPair) return __float2half2_rn(0.0f); else return 0.0f; };
+    const auto add = [](R a, R b) { if constexpr (kPair) return __hadd2(a, b); else return a + b; };
+    const auto term = [&](int i) {
+        if constexpr (kPair) return sm.u.term2[PF_IDX(i, kRoiMax / 2)];
+        else return HalfOps<H>::to_f(sm.u.term[PF_IDX(i, kRoiMax)]);
+    };
+    for (int y0 = 0; y0 < wh; y0 += band) {
+        const int nb = wh - y0 < band ? wh - y0 : band, nr = nb + 2 * r;
+        for (int i = tid; i < nr * pw; i += kThreads) {
+            const int yy = i / pw, hp = i - yy * pw;
+            const int base = (y0 + yy) * rw + (kPair ? 2 * hp : hp) + r;
+            for (int c = 0; c < ncls; c += 4) {
+                const int h0 = T.chw[c], h1 = T.chw[c + 1], h2 = T.chw[c + 2], h3 = T.chw[c + 3];
+                R a0 = zero(), a1 = a0, a2 = a0, a3 = a0;
+#pragma unroll 4
+                for (int dx = -h0; dx <= h0; ++dx) {
+                    const R t = term(base + dx);
+                    const int ad = dx < 0 ? -dx : dx;
+                    a0 = add(a0, t);
+                    if (ad <= h1) a1 = add(a1, t);
+                    if (ad <= h2) a2 = add(a2, t);
+                    if (ad <= h3) a3 = add(a3, t);
+                }
+                R *o = rows + (c * nr + yy) * pw + hp;
+                o[0] = a0;
+                if (h1 >= 0) o[nr * pw] = a1;
+                if (h2 >= 0) o[2 * nr * pw] = a2;
+                if (h3 >= 0) o[3 * nr * pw] = a3;
+            }
+        }
+        __syncthreads();
+        for (int i = tid; i < nb * pw; i += kThreads) {
+            const int cy = i / pw, hp = i - cy * pw;
+            R acc = zero();
+#pragma unroll 4
+            for (int k = 0; k <= 2 * r; ++k) acc = add(acc, rows[PF_IDX((T.rc[k] * nr + cy + k) * pw + hp, kRowWords)]);
+            if constexpr (kPair) {
+                const int cx = 2 * hp, c = (y0 + cy) * ww + cx;
+                sm.table[PF_IDX(c, kTableMax)] = __low2half(acc);
+                if (cx + 1 < ww) sm.table[PF_IDX(c + 1, kTableMax)] = __high2half(acc);
+            } else {
+                sm.table[PF_IDX((y0 + cy) * ww + hp, kTableMax)] = HalfOps<H>::from_f(acc);
+            }
+        }
+        if (y0 + band < wh) __syncthreads();   // (the next band rewrites the row sums)
+    }
+}
 
 // One tile of a launch in mode kMode (trackers of the other modes are skipped).
 template <int P, int kMode>
@@ -1105,7 +1177,6 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
         fv.pitch = sm.fr.pitch;
     }
     const int r = fv.r;
-    for (int i = tid; i <= 2 * r; i += kThreads) sm.w[i] = static_cast<int8_t>(row_half_width(r, i - r));
 
     using H = typename std::conditional<Tr::kHalf, pos_t, __half>::type;
 
@@ -1376,10 +1447,10 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
                 const int px = gx0 + c % gw, py = gy0 + c / gw;
                 uint32_t payload;
                 if constexpr (Tr::kHalf) {
-                    const H v = half_lik<H>(T).warp_at(fv, px, py);
+                    const H v = half_lik<H>(T).warp_at(fv, T.w, px, py);
                     payload = static_cast<uint32_t>(*reinterpret_cast<const unsigned short *>(&v));
                 } else {
-                    payload = warp_disk_sum(fv, px, py);
+                    payload = warp_disk_sum(fv, T.w, px, py);
                 }
                 if (lane == 0) st_relaxed_u64(&T.gtab[PF_IDX(c, kTableMax)], gtag | payload);
             }
@@ -1442,7 +1513,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
     const acc_t den = kF64 ? static_cast<acc_t>(T.den) : static_cast<acc_t>(T.denf);
 
     // ------------------------------------------------------------ 1c. likelihood table
-    if (kMode != kModeCdf && cells > 0 && !gt) {
+    if constexpr (kMode != kModeCdf) if (cells > 0 && !gt) {
         // stage the frame region the window's templates cover (clamped to the frame);
         // warp w takes rows w, w + kWarps, ...; its lanes walk the row
         const int rx0 = wx0 - r, ry0 = wy0 - r, rw = ww + 2 * r, rh = wh + 2 * r;
@@ -1488,7 +1559,30 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             }
         }
         __syncthreads();
-        if (paired) {
+        bool by_rows = false;
+        if constexpr (Tr::kHalf) {
+            const int pw = paired ? (ww + 1) >> 1 : (ww > 0 ? ww : 1);   // words a row
+            // (the tracker-table mode has no memory for them: its map is in use; a tile of its
+            // own is the exception there)
+            int band = (kMode == kModeStep ? kRowWords : kMapMax / 2) / (T.ncls * pw) - 2 * r;
+            if (band > wh) band = wh;
+            // Row sums where they are the shorter way, block passes counted: about 10 issue slots
+            // a term of a row (four classes at once) and 5 a row of a cell, against 4 a template
+            // pixel (a dependent load and addition) and 10 a row, every cell by itself.  So by
+            // rows except where the cells fill one pass and their rows several
+            const int by_row = ((rh * pw - 1) / kThreads + 1) * (10 * T.row_terms + 30) +
+                               ((wh * pw - 1) / kThreads + 1) * 5 * (2 * r + 1);
+            const int by_cell = ((wh * pw - 1) / kThreads + 1) * (4 * T.D + 10 * (2 * r + 1));
+            by_rows = (paired || !hk.half_acc) && (band == wh || band >= 4) && by_row < by_cell &&
+                      (kMode == kModeStep || (kMode == kModePull && !T.dbg_anc));
+            if (by_rows) {
+                if constexpr (P == 2) {
+                    if (paired) table_by_rows<P, kMode, true>(sm, rw, pw, ww, wh, band, st);
+                }
+                if (!paired) table_by_rows<P, kMode, false>(sm, rw, pw, ww, wh, band, st);
+            }
+        }
+        if (paired && !by_rows) {
             // two neighbouring cells (cx, cx + 1) a thread, one in each half2 lane: each lane
             // performs its cell's additions of from_terms in the same order (an odd row's
             // last pair computes a cell past the row and drops it)
@@ -1497,7 +1591,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
                 const int cy = pi / hpr, cx = 2 * (pi - cy * hpr);
                 __half2 acc = __float2half2_rn(0.0f);
                 for (int i = 0; i <= 2 * r; ++i) {
-                    const int hw = sm.w[i];
+                    const int hw = sm.trk.w[i];
                     const int b = (cy + i) * rw + cx + r;
                     __half2 rs = __float2half2_rn(0.0f);
 #pragma unroll 4
@@ -1512,15 +1606,15 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             }
         }
         const int wdiv = kMode != kModeCdf ? ww : 1;    // (no table in the CDF kernel)
-        for (int c = paired ? cells : tid, cy = tid / wdiv, cx = tid - (tid / wdiv) * wdiv; c < cells; c += kThreads) {
+        for (int c = paired || by_rows ? cells : tid, cy = tid / wdiv, cx = tid - (tid / wdiv) * wdiv; c < cells; c += kThreads) {
             if constexpr (Tr::kHalf) {
-                sm.table[PF_IDX(c, kTableMax)] = hk.from_terms(sm.u.term, rw, sm.w, r, cx, cy);
+                sm.table[PF_IDX(c, kTableMax)] = hk.from_terms(sm.u.term, rw, sm.trk.w, r, cx, cy);
             } else {
                 uint32_t ssum = 0;
 #pragma unroll 4
                 for (int i = 0; i <= 2 * r; ++i) {
                     const uint16_t *p = sm.u.pre + (cy + i) * (rw + 1) + cx + r;
-                    const int hw = sm.w[i];
+                    const int hw = sm.trk.w[i];
                     ssum += static_cast<uint32_t>(static_cast<uint16_t>(p[hw + 1] - p[-hw]));
                 }
                 sm.table[PF_IDX(c, kTableMax)] = lik_from_sum<acc_t>(ssum, c1, c2D, den);
@@ -1800,13 +1894,13 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             acc_t L0 = v0 && in0 ? sm.table[cy0 * ww + cx0] : static_cast<acc_t>(0);
             acc_t L1 = v1 && in1 ? sm.table[cy1 * ww + cx1] : static_cast<acc_t>(0);
             if constexpr (kMode == kModeStepBig) {   // (the tracker's table takes every draw: rarer still)
-                if (v0 && !in0) L0 = lik_from_sum<acc_t>(disk_sum(fv, sm.w, pixel_of(x0), pixel_of(y0)), c1, c2D, den);
-                if (v1 && !in1) L1 = lik_from_sum<acc_t>(disk_sum(fv, sm.w, pixel_of(x1), pixel_of(y1)), c1, c2D, den);
+                if (v0 && !in0) L0 = lik_from_sum<acc_t>(disk_sum(fv, sm.trk.w, pixel_of(x0), pixel_of(y0)), c1, c2D, den);
+                if (v1 && !in1) L1 = lik_from_sum<acc_t>(disk_sum(fv, sm.trk.w, pixel_of(x1), pixel_of(y1)), c1, c2D, den);
             } else {
                 const int miss = (v0 && !in0 ? 1 : 0) | (v1 && !in1 ? 2 : 0);
                 const unsigned act = __activemask();
                 if (__any_sync(act, miss != 0))
-                    direct_likelihoods<P>(T, fv, sm.w, act, miss, pixel_of(x0), pixel_of(y0), pixel_of(x1), pixel_of(y1), L0, L1);
+                    direct_likelihoods<P>(T, fv, sm.trk.w, act, miss, pixel_of(x0), pixel_of(y0), pixel_of(x1), pixel_of(y1), L0, L1);
             }
             if (v0 && v1) {
                 if constexpr (sizeof(acc_t) == 8) {
@@ -1859,13 +1953,13 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             H l0 = in0 ? sm.table[cy0 * ww + cx0] : OPS::from_f(0.0f);
             H l1 = in1 ? sm.table[cy1 * ww + cx1] : OPS::from_f(0.0f);
             if constexpr (kMode == kModeStepBig) {   // (the tracker's table takes every draw: rarer still)
-                if (v0 && !in0) l0 = hk.at(fv, sm.w, axi + pixel_of(OPS::lo(ox)), ayi + pixel_of(OPS::lo(oy)));
-                if (v1 && !in1) l1 = hk.at(fv, sm.w, axi + pixel_of(OPS::hi(ox)), ayi + pixel_of(OPS::hi(oy)));
+                if (v0 && !in0) l0 = hk.at(fv, sm.trk.w, axi + pixel_of(OPS::lo(ox)), ayi + pixel_of(OPS::lo(oy)));
+                if (v1 && !in1) l1 = hk.at(fv, sm.trk.w, axi + pixel_of(OPS::hi(ox)), ayi + pixel_of(OPS::hi(oy)));
             } else {
                 const int miss = (v0 && !in0 ? 1 : 0) | (v1 && !in1 ? 2 : 0);
                 const unsigned act = __activemask();
                 if (__any_sync(act, miss != 0))
-                    direct_likelihoods<P>(T, fv, sm.w, act, miss, axi + pixel_of(OPS::lo(ox)), ayi + pixel_of(OPS::lo(oy)),
+                    direct_likelihoods<P>(T, fv, sm.trk.w, act, miss, axi + pixel_of(OPS::lo(ox)), ayi + pixel_of(OPS::lo(oy)),
                                           axi + pixel_of(OPS::hi(ox)), ayi + pixel_of(OPS::hi(oy)), l0, l1);
             }
             if (v0 && v1) {
