@@ -36,14 +36,7 @@ __device__ __forceinline__ float uniform_f32(uint32_t w) {
 }
 __device__ __forceinline__ double uniform_f64(uint32_t w) { return static_cast<double>(uniform_f32(w)); }
 
-// Box-Muller: two N(0,1) draws from two uniforms.
-__device__ __forceinline__ void box_muller(double ua, double ub, double &nx, double &ny) {
-    const double rad = sqrt(-2.0 * log(ua));
-    double s, c;
-    sincospi(2.0 * ub, &s, &c);
-    nx = rad * c;
-    ny = rad * s;
-}
+// Box-Muller: two N(0,1) draws from two uniforms (FP64: box_muller_table in pf_ref64.cuh).
 __device__ __forceinline__ void box_muller(float ua, float ub, float &nx, float &ny) {
     const float rad = sqrtf(-2.0f * logf(ua));
     float s, c;

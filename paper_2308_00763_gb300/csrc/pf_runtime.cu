@@ -344,6 +344,7 @@ static pf_status engine_init(Engine &e, const pf_config *cfgs, int n, void *stre
         if (tabs[s]->n > 0)
             err = cudaMemcpyAsync(tabs[s]->d, atab[s].data(), sizeof(int32_t) * atab[s].size(), cudaMemcpyHostToDevice,
                                   e.stream);
+    if (err == cudaSuccess && step_prepare(e.prec, e.stream) != 0) err = cudaErrorUnknown;
     if (err == cudaSuccess) err = cudaMemsetAsync(e.d_ticket, 0, sizeof(uint32_t), e.stream);
     memcpy(e.h_init_pinned, st.data(), sizeof(TrackerState) * n);
     for (int i = 0; i < n && err == cudaSuccess; ++i)

@@ -52,6 +52,7 @@
 
 #include "pf_device.cuh"
 #include "pf_internal.h"
+#include "pf_ref64.cuh"
 
 // The pull kernel's offspring have no likelihood table (window width 0), so its bounds
 // tests against the window compare unsigned values with a constant 0.
@@ -206,7 +207,7 @@ __device__ void wait_partial(const TilePartial *p, uint64_t tag, TrackerState *s
 // exp(d) for d <= 0 with the two exact shortcuts: exp(0) = 1, and 0 below the point
 // where the precision underflows to zero anyway.
 __device__ __forceinline__ double exp_le0(double d) {
-    return d == 0.0 ? 1.0 : (d < -746.0 ? 0.0 : exp(d));
+    return exp_table_takes(d) ? exp_table(d) : (d < -746.0 ? 0.0 : exp(d));
 }
 __device__ __forceinline__ float exp_le0(float d) {
     return d == 0.0f ? 1.0f : (d < -104.0f ? 0.0f : expf(d));
@@ -248,10 +249,12 @@ __device__ __forceinline__ void stats_add2(Stats<A> &a, bool v0, A L0, A dx0, A 
     const A l0 = v0 ? L0 : neg_inf<A>(), l1 = v1 ? L1 : neg_inf<A>();
     const A mx = l0 > l1 ? l0 : l1;
     const A nm = mx > a.m ? mx : a.m;
-    const A sc = (nm == neg_inf<A>()) ? static_cast<A>(1)
-                                      : ((a.m == neg_inf<A>()) ? static_cast<A>(0) : wexp<F>(a.m - nm));
-    a.s *= sc; a.sx *= sc; a.sy *= sc;
-    a.m = nm;
+    if (sizeof(A) == 4 || nm != a.m) {   // (a factor of 1 costs FP64 more than a branch)
+        const A sc = (nm == neg_inf<A>()) ? static_cast<A>(1)
+                                          : ((a.m == neg_inf<A>()) ? static_cast<A>(0) : wexp<F>(a.m - nm));
+        a.s *= sc; a.sx *= sc; a.sy *= sc;
+        a.m = nm;
+    }
     const A e0 = v0 ? wexp<F>(l0 - a.m) : static_cast<A>(0);
     const A e1 = v1 ? wexp<F>(l1 - a.m) : static_cast<A>(0);
     a.s += e0 + e1;
@@ -1877,8 +1880,8 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             }
             acc_t n0x, n0y, n1x, n1y;
             if constexpr (sizeof(acc_t) == 8) {
-                box_muller(uniform_f64(wd.x), uniform_f64(wd.y), n0x, n0y);
-                box_muller(uniform_f64(wd.z), uniform_f64(wd.w), n1x, n1y);
+                box_muller_table(wd.x, wd.y, n0x, n0y);
+                box_muller_table(wd.z, wd.w, n1x, n1y);
             } else {
                 box_muller(uniform_f32(wd.x), uniform_f32(wd.y), n0x, n0y);
                 box_muller(uniform_f32(wd.z), uniform_f32(wd.w), n1x, n1y);
@@ -2157,6 +2160,50 @@ int slots_of(int precision) {
     return g;
 }
 }  // namespace
+
+// The FP64 tables, each entry rounded once from extended precision.
+static Ref64Tables::Ln split_ln(float c, long double v) {
+    const long double hi = rintl(v * 4398046511104.0L) / 4398046511104.0L;   // a multiple of 2^-42
+    return Ref64Tables::Ln{c, static_cast<float>(v - hi), static_cast<double>(hi)};
+}
+static bool fill_ref64_tables(Ref64Tables &t) {
+    const long double pi = 3.14159265358979323846264338327950288L, ln2 = 0.693147180559945309417232121458176568L;
+    for (int i = 0; i < 2048; ++i) {
+        t.turn_hi[i] = double2{static_cast<double>(cosl(pi * i / 4096)), static_cast<double>(sinl(pi * i / 4096))};
+        t.turn_lo[i] = double2{static_cast<double>(cosl(pi * i / 8388608)), static_cast<double>(sinl(pi * i / 8388608))};
+        const long double e = exp2l(static_cast<long double>(i) / 2048);
+        t.ex[i].x = static_cast<double>(e);
+        t.ex[i].y = static_cast<double>(e - t.ex[i].x);
+    }
+    for (int i = 0; i < 32; ++i) t.eln2[i] = split_ln(0.0f, -ln2 * i);
+    for (int j = 0; j < 1024; ++j) {
+        // the last interval takes c = 1/2, so that ln u keeps its relative accuracy next to u = 1
+        const float c = j == 1023 ? 0.5f : static_cast<float>(1.0 / (1.0 + (j + 0.5) / 1024));
+        const long double cl = c;
+        t.ln[j] = split_ln(c, -logl(j >= kLnUpper ? 2 * cl : cl));
+    }
+    return true;
+}
+static const Ref64Tables &ref64_tables() {
+    static Ref64Tables t;
+    static const bool filled = fill_ref64_tables(t);
+    (void)filled;
+    return t;
+}
+
+int step_prepare(int precision, void *stream) {
+    if (precision != 0) return 0;
+    static std::atomic<int> ready[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return -1; }
+    if (dev >= 0 && dev < 64 && ready[dev].load(std::memory_order_acquire)) return 0;
+    const cudaStream_t s = static_cast<cudaStream_t>(stream);
+    cudaError_t err = cudaMemcpyToSymbolAsync(g_ref64, &ref64_tables(), sizeof(Ref64Tables), 0, cudaMemcpyHostToDevice, s);
+    if (err == cudaSuccess) err = cudaStreamSynchronize(s);
+    if (err != cudaSuccess) { cudaGetLastError(); return -1; }
+    if (dev >= 0 && dev < 64) ready[dev].store(1, std::memory_order_release);
+    return 0;
+}
 
 int step_tile_size(int precision, int64_t n) {
     const int64_t slots = slots_of(precision);

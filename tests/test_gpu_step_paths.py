@@ -1,0 +1,115 @@
+"""Routes of the step that ordinary videos seldom take, against the oracle: every particle outside
+any likelihood table (the direct route), tables built from row sums in bands, the FP64 draws
+of a whole frame, the multinomial search at the edges of its levels, and Gumbel-max draws over
+flat weights (no particle can be ruled out).
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2308_00763_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pf():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2308_00763_gb300 as m
+    m.lib(build_if_missing=True)
+    return m
+
+
+def _cuda(frames):
+    import torch
+    return torch.from_numpy(frames).cuda()
+
+
+def _check_likelihoods(pf, f, prec, frame, r, flags=0):
+    st = f.get_state()
+    half = prec in ("f16", "bf16")
+    x = st["x"] + (st["anchor_x"] if half else 0.0)
+    y = st["y"] + (st["anchor_y"] if half else 0.0)
+    if half:   # the same operations, each rounded once: bit for bit
+        kind = "f16acc32" if prec == "f16" and flags & pf.PF_FLAG_ACCUM32 else prec
+        assert np.array_equal(st["L"], oracle.likelihood_half(x, y, frame, r, kind))
+    elif prec == "ref64":
+        assert np.array_equal(st["L"], oracle.likelihood_all(x, y, frame, r))
+    else:
+        np.testing.assert_allclose(st["L"], oracle.likelihood_all(x, y, frame, r), rtol=2 ** -23, atol=1e-4)
+
+
+@pytest.mark.parametrize("prec,accum32", [("ref64", 0), ("f32", 0), ("f16", 0), ("f16", 1), ("bf16", 0)])
+@pytest.mark.parametrize("r", [0, 5, 40])
+def test_direct_route_of_every_particle(pf, prec, accum32, r):
+    """Draws of 40 px: no window fits a table, so every lane's two particles go to the frame
+    (whole warps, partial warps at the tile's end and the straddling pairs)."""
+    v = synth.make_video(200, 150, 3, 6, noise=8.0, seed=21)
+    flags = pf.PF_FLAG_DEBUG_ARRAYS | (pf.PF_FLAG_ACCUM32 if accum32 else 0)
+    f = pf.Filter(v.W, v.H, 1027, r, prec, init=tuple(v.centres[0]), seed=8, sigma=(40.0, 40.0), flags=flags)
+    f.run(_cuda(v.frames))
+    assert np.all(f.debug(2)[:, 2] == 0)
+    _check_likelihoods(pf, f, prec, v.frames[-1], r, flags)
+    f.close()
+
+
+@pytest.mark.parametrize("prec,accum32", [("f16", 0), ("f16", 1), ("bf16", 0)])
+@pytest.mark.parametrize("r", [1, 7, 14, 20])
+def test_tables_by_row_sums_and_bands(pf, prec, accum32, r):
+    v = synth.make_video(160, 140, 3, r, noise=8.0, seed=22, c0=(60.0, 60.0))
+    flags = pf.PF_FLAG_DEBUG_ARRAYS | (pf.PF_FLAG_ACCUM32 if accum32 else 0)
+    for resampler in ("systematic", "multinomial"):
+        f = pf.Filter(v.W, v.H, 3000, r, prec, init=tuple(v.centres[0]), seed=8, flags=flags, resampler=resampler)
+        f.run(_cuda(v.frames))
+        assert np.all(f.debug(2)[:, 2] > 0)
+        _check_likelihoods(pf, f, prec, v.frames[-1], r, flags)
+        f.close()
+
+
+def test_fp64_draws_of_a_frame(pf):
+    """2^20 normal pairs around the origin.  Radii are below 5.77, within 1 ulp (9e-16) on either
+    side; the step's sine and cosine are within 1.7e-16, the oracle's within 1.2e-16 of those of
+    its angle, whose product 2 pi u is off by up to 7e-16: 5.77 x 9.9e-16 + 2 x 9e-16 < 8e-15."""
+    v = synth.make_video(64, 64, 1, 3, noise=5.0, seed=23)
+    n = 1 << 20
+    f = pf.Filter(v.W, v.H, n, 3, "ref64", init=(0.0, 0.0), seed=24)
+    f.run(_cuda(v.frames))
+    st = f.get_state()
+    f.close()
+    nx, ny = oracle.normals(24, 0, n)
+    assert np.abs(st["x"] - nx).max() <= 8e-15 and np.abs(st["y"] - ny).max() <= 8e-15
+
+
+@pytest.mark.parametrize("prec,n", [("f32", n) for n in (7, 8, 9, 63, 64, 65, 511, 4097, (1 << 20) + 9)] +
+                         [("ref64", 65), ("ref64", 70001), ("f16", 130), ("f16", 700001)])
+def test_multinomial_search_at_the_edges_of_its_levels(pf, prec, n):
+    v = synth.make_video(128, 128, 3, 5, noise=5.0, seed=25)
+    f = pf.Filter(v.W, v.H, n, 5, prec, init=tuple(v.centres[0]), seed=26, flags=pf.PF_FLAG_DEBUG_ARRAYS,
+                  resampler="multinomial")
+    f.run(_cuda(v.frames))
+    anc, c = f.debug(0).astype(np.int64), f.debug(1).astype(np.float64)
+    f.close()
+    want = oracle.resample_multinomial(c, oracle.stratified_offsets(26, v.T - 2, n), "f64" if prec == "ref64" else "f32")
+    assert np.array_equal(anc, want)
+
+
+@pytest.mark.parametrize("prec", ["ref64", "f32", "f16"])
+def test_gumbel_over_flat_weights(pf, prec):
+    """A frame of one level: every likelihood is the same, no particle can be ruled out."""
+    frames = np.full((2, 64, 64), 100, np.uint8)
+    n = 1500
+    f = pf.Filter(64, 64, n, 3, prec, init=(32.0, 32.0), seed=27, flags=pf.PF_FLAG_DEBUG_ARRAYS, resampler="gumbel")
+    f.step(_cuda(frames)[0])
+    like = f.get_state()["L"].astype(np.float64)
+    assert np.all(like == like[0])
+    f.step(_cuda(frames)[1])
+    anc = f.debug(0).astype(np.int64)
+    f.close()
+    want = oracle.resample_gumbel(like, 27, 0, 0, "f64" if prec == "ref64" else "f32")
+    bad = np.nonzero(anc != want)[0]   # (near ties of the two sides' logarithms)
+    assert bad.size <= 2
+    for j in bad:
+        g = oracle.gumbel_variates(27, 0, int(j), n)
+        assert abs(g[want[j]] - g[anc[j]]) <= (1e-12 if prec == "ref64" else 1e-5) * max(1.0, abs(like[0]))
