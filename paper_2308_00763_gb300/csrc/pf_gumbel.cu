@@ -11,13 +11,26 @@
 // the sum is taken in the filter's weight precision: FP64 for REF64, FP32 for the others
 // (L widened from its stored type).  Ties go to the smallest k.
 //
+// Most of the N^2 variates cannot win, and are refused without their two logarithms:
+//   - g_jk lies in [-2.82, 16.64] (u has 24 bits), and the particle of the largest L enters
+//     every offspring's argmax with at least max L - 2.82, so a particle below max L - 19.5
+//     never wins: the CTA lists the quads with a particle above that line and draws for those
+//     alone.  (max L is taken over the CTA's own pass over L, whatever state was loaded.)
+//   - -ln u >= 1 - u gives g <= -ln(1 - u), so a variate beats the CTA's best b_j so far only
+//     if (1 - u) exp(b_j - max L) <= exp(L_k - max L): one product in FP32 against two
+//     logarithms, with a margin (1e-3 and 4e-6 max |L| relative) above the rounding of both sides.
+// Whoever passes is evaluated as before, so the argmax and its ties are the same.
+//
 // Layout: CTA b takes kGumbelOffspring consecutive offspring of one tracker.  Its threads
-// stride over the particle quads q (particles 4q .. 4q+3): one Philox block per (quad,
+// stride over the listed particle quads q (particles 4q .. 4q+3): one Philox block per (quad,
 // offspring) gives that offspring's four draws, the quad's four L are loaded once for all
-// of the CTA's offspring, and each thread keeps a running best per offspring (k rises
-// within a thread, so a strict comparison keeps the smallest k of equal values).  The CTA
-// then reduces each offspring's (value, index) pairs: warp shuffles, then one thread per
-// offspring over the warps' results.  The pull kernel gathers the ancestors written here.
+// of the CTA's offspring, and each thread keeps a running best per offspring (ties to the
+// smaller index).  The best of all threads, as exp(b_j - max L), is shared through shared
+// memory for the test above.  The CTA then reduces each offspring's (value, index) pairs:
+// warp shuffles, then one thread per offspring over the warps' results.  The pull kernel
+// gathers the ancestors written here.
+// Measured us a frame on the tracker's peaked weights, every variate in full -> these tests: F32
+// 8191 particles 166 -> 108, REF64 2047 543 -> 254.
 #include <math.h>
 
 #include "pf_ancestor.cuh"
@@ -47,6 +60,10 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
     constexpr int kWarps = kGumbelThreads / 32;
     __shared__ acc_t s_v[kWarps][kJ];
     __shared__ int s_k[kWarps][kJ];
+    __shared__ uint16_t s_list[kGumbelMaxN / 4];   // quads with a particle that can win
+    __shared__ unsigned int s_n;
+    __shared__ acc_t s_max[kWarps];
+    __shared__ unsigned int s_eb[kJ];              // exp(best - max L) of the CTA, float bits (>= 0)
 
     const int b = static_cast<int>(blockIdx.x);
     const int g = ancestor_tracker(G, b);
@@ -69,11 +86,52 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
         arg[jj] = N;
     }
     const int nq = (N + 3) >> 2;
-    for (int q = threadIdx.x; q < nq; q += kGumbelThreads) {
-        const int k = 4 * q;
-        acc_t l[4];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // the largest L (NaN aside) and the list of quads that can win
+    acc_t mx = -INFINITY;
+    for (int k = threadIdx.x; k < N; k += kGumbelThreads) {
+        const acc_t l = to_acc(L[k]);
+        mx = l > mx ? l : mx;
+    }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) l[i] = (k + i < N) ? to_acc(L[k + i]) : static_cast<acc_t>(-INFINITY);
+    for (int o = 16; o > 0; o >>= 1) {
+        const acc_t y = __shfl_xor_sync(0xffffffffu, mx, o);
+        mx = y > mx ? y : mx;
+    }
+    if (lane == 0) s_max[wid] = mx;
+    if (threadIdx.x == 0) s_n = 0u;
+    if (threadIdx.x < kJ) s_eb[threadIdx.x] = 0u;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) mx = s_max[w] > mx ? s_max[w] : mx;
+    const bool finite = mx - mx == static_cast<acc_t>(0);   // else every quad is evaluated in full
+    const acc_t line = mx - static_cast<acc_t>(19.5) - static_cast<acc_t>(1e-5) * (mx < 0 ? -mx : mx);
+    for (int q0 = 0; q0 < nq; q0 += kGumbelThreads) {
+        const int q = q0 + static_cast<int>(threadIdx.x), k = 4 * q;
+        bool keep = false;
+        if (q < nq) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) keep = keep || (k + i < N && (!finite || to_acc(L[k + i]) >= line));
+        }
+        const uint32_t mask = __ballot_sync(0xffffffffu, keep);
+        unsigned int at = 0;
+        if (lane == 0 && mask) at = atomicAdd(&s_n, static_cast<unsigned int>(__popc(mask)));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (keep) s_list[at + __popc(mask & ((1u << lane) - 1u))] = static_cast<uint16_t>(q);
+    }
+    __syncthreads();
+    const int nl = static_cast<int>(s_n);
+    const float mxf = static_cast<float>(mx);
+    const float margin = 1.001f + 4e-6f * fabsf(mxf);
+    for (int p = threadIdx.x; p < nl; p += kGumbelThreads) {
+        const int q = s_list[p], k = 4 * q;
+        acc_t l[4];
+        float el[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            l[i] = (k + i < N) ? to_acc(L[k + i]) : static_cast<acc_t>(-INFINITY);
+            el[i] = margin * __expf(static_cast<float>(l[i] - mx));
+        }
 #pragma unroll
         for (int jj = 0; jj < kJ; ++jj) {
             const int j = j0 + jj;
@@ -82,19 +140,22 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
                                                      trk_id),
                                           key_lo, key_hi);
             const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+            const float eb = __uint_as_float(*reinterpret_cast<volatile unsigned int *>(&s_eb[jj]));
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
+                // (not taken when either side is NaN: evaluated in full)
+                if (finite && (1.0f - uniform_f32(ws[i])) * eb > el[i]) continue;
                 if (k + i < N) {
                     const acc_t v = l[i] + gumbel_of(ws[i], acc_t{});
-                    if (v > best[jj]) {
+                    if (v > best[jj] || (v == best[jj] && k + i < arg[jj] && arg[jj] < N)) {
                         best[jj] = v;
                         arg[jj] = k + i;
+                        if (finite) atomicMax(&s_eb[jj], __float_as_uint(__expf(static_cast<float>(v - mx))));
                     }
                 }
             }
         }
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int jj = 0; jj < kJ; ++jj) {
         acc_t v = best[jj];

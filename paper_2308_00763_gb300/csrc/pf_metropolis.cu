@@ -28,9 +28,6 @@
 namespace pfk {
 namespace {
 
-__device__ __forceinline__ double log_uniform(uint32_t w, double) { return log(uniform_f64(w)); }
-__device__ __forceinline__ float log_uniform(uint32_t w, float) { return logf(uniform_f32(w)); }
-
 template <int P>
 __global__ void __launch_bounds__(kMetropolisThreads) metropolis_kernel(const AncestorLaunch G) {
     using lik_t = typename Prec<P>::lik_t;
@@ -74,7 +71,7 @@ __global__ void __launch_bounds__(kMetropolisThreads) metropolis_kernel(const An
         }
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            if (s + q < B && log_uniform(wu[q], acc_t{}) <= lq[q] - lk) {
+            if (s + q < B && log_uniform_le<acc_t>(wu[q], lq[q] - lk)) {
                 k = kq[q];
                 lk = lq[q];
             }

@@ -29,9 +29,6 @@
 namespace pfk {
 namespace {
 
-__device__ __forceinline__ double log_uniform(uint32_t w, double) { return log(uniform_f64(w)); }
-__device__ __forceinline__ float log_uniform(uint32_t w, float) { return logf(uniform_f32(w)); }
-
 template <int P>
 __global__ void __launch_bounds__(kRejectionThreads) rejection_kernel(const AncestorLaunch G) {
     using lik_t = typename Prec<P>::lik_t;
@@ -83,7 +80,7 @@ __global__ void __launch_bounds__(kRejectionThreads) rejection_kernel(const Ance
         int dec = -1;
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-            if (dec < 0 && i + q < R && (log_uniform(wu[q], acc_t{}) <= lq[q] - M || i + q + 1 >= R)) dec = q;
+            if (dec < 0 && i + q < R && (log_uniform_le<acc_t>(wu[q], lq[q] - M) || i + q + 1 >= R)) dec = q;
         if (dec >= 0) {
             int kd = kq[0];
 #pragma unroll
