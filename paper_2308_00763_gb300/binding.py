@@ -819,8 +819,9 @@ class Server:
         if on_dev:
             q[1].append((q[0], keep))
         q[0] += 1
-        done = pf_server_frames_done(self.h, sid)
-        q[1] = [(i, t) for i, t in q[1] if i >= done]
+        if len(q[1]) > 2 * self.cfg.queue_depth:   # (at most queue_depth are still in use)
+            done = pf_server_frames_done(self.h, sid)
+            q[1] = [(i, t) for i, t in q[1] if i >= done]
         return True
 
     def tick(self):

@@ -235,6 +235,12 @@ int step_grid_size(int precision, int total_tiles);
 int step_tile_size(int precision, int64_t n);
 int launch_debug_philox(const uint32_t *d_ctrs, int64_t n, uint64_t seed, uint32_t *d_out,
                         void *stream);
+// Back to frame 0: every tracker's state from init[i] except the launch counter (epoch) and the
+// status word, and its lookback descriptors cleared (their tags are launch counters modulo
+// 65535: cleared words can never look current).  max_tiles: the most tiles of any tracker.
+int launch_reset(const TrackerDev *trk, const TrackerState *init, int n, int max_tiles, void *stream);
+// out[2 i .. 2 i + 1] = entry frame mod est_cap of tracker i's estimate ring.
+int launch_gather_estimates(const TrackerDev *trk, int n, int64_t frame, double *out, void *stream);
 int launch_wait_probe(void *d_desc, void *d_state, uint32_t limit, void *stream);
 
 }  // namespace pfk

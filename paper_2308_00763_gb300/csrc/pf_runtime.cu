@@ -117,7 +117,12 @@ struct Engine {
     int ctas_cap = 0;                  // CTAs per SM (0: as many as fit)
     pf_status sticky = PF_OK;
     uint8_t *d_frame_buf = nullptr;    // single tracker: staging of host frames
-    TrackerState *h_init_pinned = nullptr;  // initial state of every tracker (pf_reset)
+    // initial state of every tracker: uploaded once, copied into the states by the reset kernel
+    TrackerState *d_init = nullptr;    // in the arena
+    // one pinned block that results are read back into: [n] states, then [n] gathered estimates
+    TrackerState *h_states = nullptr;
+    double *h_gather = nullptr;
+    double *d_gather = nullptr;        // in the arena
     cudaEvent_t frames_copied = nullptr;     // the pinned frame table may be rewritten after it
     cudaStream_t capture_stream = nullptr;   // private stream used to capture step graphs
     std::vector<std::pair<int32_t, cudaGraphExec_t>> graphs;   // count consecutive steps, replayed
@@ -174,8 +179,8 @@ static void engine_free(Engine &e) {
     cudaFree(e.d_arena);
     cudaFree(e.d_frame_buf);
     if (e.h_frames_pinned) cudaFreeHost(e.h_frames_pinned);
-    if (e.h_init_pinned) cudaFreeHost(e.h_init_pinned);
-    e.h_init_pinned = nullptr;
+    if (e.h_states) cudaFreeHost(e.h_states);
+    e.h_states = nullptr; e.h_gather = nullptr; e.d_init = nullptr; e.d_gather = nullptr;
     e.d_trk = nullptr; e.d_frames = nullptr; e.d_tile_trk = nullptr; e.d_ticket = nullptr;
     e.gumbel.d = nullptr; e.metro.d = nullptr; e.rej.d = nullptr;
     e.d_arena = nullptr; e.d_frame_buf = nullptr; e.h_frames_pinned = nullptr;
@@ -206,6 +211,7 @@ static pf_status engine_init(Engine &e, const pf_config *cfgs, int n, void *stre
     std::vector<Off> off(n);
     // the trackers' states form one array (the kernel indexes it by tracker)
     const size_t states_off = a.take(sizeof(TrackerState) * n);
+    const size_t init_off = a.take(sizeof(TrackerState) * n), gather_off = a.take(sizeof(double) * 2 * n);
     // Tiles are numbered per kernel family: the step kernel's trackers first, then the
     // pull kernel's (multinomial, Gumbel-max, Metropolis, rejection), so no launch carries
     // tiles it skips.  The ancestor kernels number their CTAs per scheme.
@@ -286,7 +292,8 @@ static pf_status engine_init(Engine &e, const pf_config *cfgs, int n, void *stre
         if (tabs[s]->n > 0) err = cudaMalloc(reinterpret_cast<void **>(&tabs[s]->d), sizeof(int32_t) * atab[s].size());
     if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&e.d_ticket), sizeof(uint32_t));
     if (err == cudaSuccess) err = cudaMallocHost(reinterpret_cast<void **>(&e.h_frames_pinned), sizeof(FrameRef) * n);
-    if (err == cudaSuccess) err = cudaMallocHost(reinterpret_cast<void **>(&e.h_init_pinned), sizeof(TrackerState) * n);
+    if (err == cudaSuccess)
+        err = cudaMallocHost(reinterpret_cast<void **>(&e.h_states), (sizeof(TrackerState) + 2 * sizeof(double)) * n);
     if (err == cudaSuccess) err = cudaEventCreateWithFlags(&e.frames_copied, cudaEventDisableTiming);
     if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&e.capture_stream, cudaStreamNonBlocking);
     if (err == cudaSuccess && stage_frames) {
@@ -346,10 +353,14 @@ static pf_status engine_init(Engine &e, const pf_config *cfgs, int n, void *stre
                                   e.stream);
     if (err == cudaSuccess && step_prepare(e.prec, e.stream) != 0) err = cudaErrorUnknown;
     if (err == cudaSuccess) err = cudaMemsetAsync(e.d_ticket, 0, sizeof(uint32_t), e.stream);
-    memcpy(e.h_init_pinned, st.data(), sizeof(TrackerState) * n);
-    for (int i = 0; i < n && err == cudaSuccess; ++i)
-        err = cudaMemcpyAsync(e.h_trk[i].state, &e.h_init_pinned[i], sizeof(TrackerState), cudaMemcpyHostToDevice,
-                              e.stream);
+    e.h_gather = reinterpret_cast<double *>(e.h_states + n);
+    e.d_init = reinterpret_cast<TrackerState *>(e.d_arena + init_off);
+    e.d_gather = reinterpret_cast<double *>(e.d_arena + gather_off);
+    memcpy(e.h_states, st.data(), sizeof(TrackerState) * n);
+    if (err == cudaSuccess)
+        err = cudaMemcpyAsync(e.d_init, e.h_states, sizeof(TrackerState) * n, cudaMemcpyHostToDevice, e.stream);
+    if (err == cudaSuccess)
+        err = cudaMemcpyAsync(e.h_trk[0].state, e.d_init, sizeof(TrackerState) * n, cudaMemcpyDeviceToDevice, e.stream);
     if (err == cudaSuccess) {
         memcpy(e.h_frames_pinned, e.h_frames.data(), sizeof(FrameRef) * n);
         err = cudaMemcpyAsync(e.d_frames, e.h_frames_pinned, sizeof(FrameRef) * n, cudaMemcpyHostToDevice, e.stream);
@@ -556,28 +567,31 @@ static pf_status engine_run_host_frames(Engine &e, const uint8_t *frames, int64_
     return PF_OK;
 }
 
-static pf_status engine_sync_status(Engine &e) {
+// Every tracker's state, and what `more` enqueues behind it, read back with one wait (a
+// blocking copy per tracker cost 8 us each); then the sticky status.
+template <typename More>
+static pf_status engine_sync_status(Engine &e, More &&more) {
     if (e.sticky != PF_OK) return e.sticky;
-    cudaError_t err = cudaStreamSynchronize(e.stream);
+    cudaError_t err = cudaMemcpyAsync(e.h_states, e.h_trk[0].state, sizeof(TrackerState) * e.n, cudaMemcpyDeviceToHost,
+                                      e.stream);
+    if (err == cudaSuccess) err = more();
+    const cudaError_t sync = cudaStreamSynchronize(e.stream);
+    if (err == cudaSuccess) err = sync;
     if (err != cudaSuccess) { cudaGetLastError(); return e.fail(PF_ERR_CUDA); }
     for (int i = 0; i < e.n; ++i) {
-        uint32_t status = 0;
-        err = cudaMemcpy(&status, &e.h_trk[i].state->status, sizeof status, cudaMemcpyDeviceToHost);
-        if (err != cudaSuccess) { cudaGetLastError(); return e.fail(PF_ERR_CUDA); }
+        const uint32_t status = e.h_states[i].status;
         if (status & kStatusTimeout) return e.fail(PF_ERR_TIMEOUT);
         if (status & kStatusBounds) return e.fail(PF_ERR_STATE);   // checked builds
     }
     return PF_OK;
 }
+static pf_status engine_sync_status(Engine &e) {
+    return engine_sync_status(e, [] { return cudaSuccess; });
+}
 
-static pf_status engine_read_frame(Engine &e, int i, int64_t idx, double *xy, double *ms) {
-    const TrackerDev &T = e.h_trk[i];
-    if (idx < 0 || idx >= e.done_frames[i] || idx < e.done_frames[i] - T.est_cap) return PF_ERR_ARG;
-    const int64_t slot = idx % T.est_cap;
-    cudaError_t err = cudaMemcpy(xy, T.est_ring + 2 * slot, 2 * sizeof(double), cudaMemcpyDeviceToHost);
-    if (err == cudaSuccess && ms) err = cudaMemcpy(ms, T.stat_ring + 2 * slot, 2 * sizeof(double), cudaMemcpyDeviceToHost);
-    if (err != cudaSuccess) { cudaGetLastError(); return e.fail(PF_ERR_CUDA); }
-    return PF_OK;
+// Whether tracker i's ring holds the estimate of frame idx.
+static bool engine_has_frame(const Engine &e, int i, int64_t idx) {
+    return idx >= 0 && idx < e.done_frames[i] && idx >= e.done_frames[i] - e.h_trk[i].est_cap;
 }
 
 // ---------------------------------------------------------------------------- C ABI
@@ -664,42 +678,46 @@ pf_status pf_run_frames(pf_filter *f, const uint8_t *frames, int64_t pitch_bytes
 pf_status pf_estimate(pf_filter *f, int64_t frame_index, double *x, double *y) {
     if (!f || !x || !y) return PF_ERR_ARG;
     Engine &e = f->e;
-    pf_status s = engine_sync_status(e);
+    const TrackerDev &T = e.h_trk[0];
+    const bool has = engine_has_frame(e, 0, frame_index);
+    const pf_status s = engine_sync_status(e, [&] {
+        return has ? cudaMemcpyAsync(e.h_gather, T.est_ring + 2 * (frame_index % T.est_cap), 2 * sizeof(double),
+                                     cudaMemcpyDeviceToHost, e.stream)
+                   : cudaSuccess;
+    });
     if (s != PF_OK) return s;
-    double xy[2];
-    s = engine_read_frame(e, 0, frame_index, xy, nullptr);
-    if (s != PF_OK) return s;
-    *x = xy[0];
-    *y = xy[1];
+    if (!has) return PF_ERR_ARG;
+    *x = e.h_gather[0];
+    *y = e.h_gather[1];
     return PF_OK;
 }
 
 pf_status pf_estimates(pf_filter *f, int64_t first, int32_t count, double *xy, double *max_and_sum) {
     if (!f || !xy || count < 0) return PF_ERR_ARG;
     Engine &e = f->e;
-    pf_status s = engine_sync_status(e);
-    if (s != PF_OK) return s;
     const TrackerDev &T = e.h_trk[0];
     const int64_t done = e.done_frames[0];
-    if (count == 0) return PF_OK;
-    if (first < 0 || first + count > done || first < done - T.est_cap) return PF_ERR_ARG;
-    // copy in at most two contiguous pieces of the ring
-    int64_t idx = first;
-    int32_t left = count;
-    while (left > 0) {
-        const int64_t slot = idx % T.est_cap;
-        int64_t run = T.est_cap - slot;
-        if (run > left) run = left;
-        cudaError_t err = cudaMemcpy(xy + 2 * (idx - first), T.est_ring + 2 * slot, run * 2 * sizeof(double),
-                                     cudaMemcpyDeviceToHost);
-        if (err == cudaSuccess && max_and_sum)
-            err = cudaMemcpy(max_and_sum + 2 * (idx - first), T.stat_ring + 2 * slot, run * 2 * sizeof(double),
-                             cudaMemcpyDeviceToHost);
-        if (err != cudaSuccess) { cudaGetLastError(); return e.fail(PF_ERR_CUDA); }
-        idx += run;
-        left -= static_cast<int32_t>(run);
-    }
-    return PF_OK;
+    const bool has = first >= 0 && first + count <= done && first >= done - T.est_cap;
+    const pf_status s = engine_sync_status(e, [&] {
+        cudaError_t err = cudaSuccess;
+        // in at most two contiguous pieces of the ring
+        int64_t idx = first;
+        for (int32_t left = has ? count : 0; left > 0 && err == cudaSuccess;) {
+            const int64_t slot = idx % T.est_cap;
+            int64_t run = T.est_cap - slot;
+            if (run > left) run = left;
+            err = cudaMemcpyAsync(xy + 2 * (idx - first), T.est_ring + 2 * slot, run * 2 * sizeof(double),
+                                  cudaMemcpyDeviceToHost, e.stream);
+            if (err == cudaSuccess && max_and_sum)
+                err = cudaMemcpyAsync(max_and_sum + 2 * (idx - first), T.stat_ring + 2 * slot, run * 2 * sizeof(double),
+                                      cudaMemcpyDeviceToHost, e.stream);
+            idx += run;
+            left -= static_cast<int32_t>(run);
+        }
+        return err;
+    });
+    if (s != PF_OK) return s;
+    return count == 0 || has ? PF_OK : PF_ERR_ARG;
 }
 
 int64_t pf_frames_done(const pf_filter *f) { return f ? f->e.done_frames[0] : -1; }
@@ -722,26 +740,11 @@ pf_status pf_get_counters(const pf_filter *f, pf_counters *out) {
     return PF_OK;
 }
 
-// Clear tracker i's lookback descriptors on the engine's stream.
-static cudaError_t clear_lookback(Engine &e, int i) {
-    const TrackerDev &T = e.h_trk[i];
-    return cudaMemsetAsync(T.look, 0, sizeof(LookbackDesc) * static_cast<size_t>(T.ntiles), e.stream);
-}
-
 pf_status pf_reset(pf_filter *f) {
     if (!f) return PF_ERR_ARG;
     Engine &e = f->e;
     if (e.sticky != PF_OK) return PF_ERR_STATE;
-    // Rewrite every field of the state except the launch counter (epoch) and the status
-    // word, and clear the lookback descriptors (their tags are launch counters modulo
-    // 65535: cleared words can never look current).
-    TrackerState *d = e.h_trk[0].state;
-    const TrackerState *h = &e.h_init_pinned[0];
-    const size_t tail = sizeof(TrackerState) - offsetof(TrackerState, M);
-    cudaError_t err = cudaMemcpyAsync(&d->t, &h->t, sizeof(int64_t), cudaMemcpyHostToDevice, e.stream);
-    if (err == cudaSuccess) err = cudaMemcpyAsync(&d->M, &h->M, tail, cudaMemcpyHostToDevice, e.stream);
-    if (err == cudaSuccess) err = clear_lookback(e, 0);
-    if (err != cudaSuccess) { cudaGetLastError(); return e.fail(PF_ERR_CUDA); }
+    if (launch_reset(e.d_trk, e.d_init, e.n, e.h_trk[0].ntiles, e.stream) != 0) return e.fail(PF_ERR_CUDA);
     e.done_frames[0] = 0;
     return PF_OK;
 }
@@ -978,21 +981,17 @@ pf_status pf_batch_get_counters(const pf_batch *b, pf_counters *out) {
 }
 
 static pf_status engine_reset(Engine &e) {
-    const size_t tail = sizeof(TrackerState) - offsetof(TrackerState, M);
     pf_status s = engine_wait_staging(e);
     if (s != PF_OK) return s;
+    int tiles = 0;
     for (int i = 0; i < e.n; ++i) {
-        TrackerState *d = e.h_trk[i].state;
-        const TrackerState *h = &e.h_init_pinned[i];
-        cudaError_t err = cudaMemcpyAsync(&d->t, &h->t, sizeof(int64_t), cudaMemcpyHostToDevice, e.stream);
-        if (err == cudaSuccess) err = cudaMemcpyAsync(&d->M, &h->M, tail, cudaMemcpyHostToDevice, e.stream);
-        if (err == cudaSuccess) err = clear_lookback(e, i);
-        if (err != cudaSuccess) { cudaGetLastError(); return e.fail(PF_ERR_CUDA); }
         // resident videos: frame 0 is again the video's first frame
         FrameRef &fr = e.h_frames_pinned[i];
         if (fr.stride && e.video_start[i]) fr.base = e.video_start[i];
         e.done_frames[i] = 0;
+        tiles = std::max(tiles, e.h_trk[i].ntiles);
     }
+    if (launch_reset(e.d_trk, e.d_init, e.n, tiles, e.stream) != 0) return e.fail(PF_ERR_CUDA);
     return engine_upload_frames(e);
 }
 
@@ -1005,19 +1004,20 @@ pf_status pf_batch_reset(pf_batch *b) {
 pf_status pf_batch_estimates(pf_batch *b, int64_t frame_index, double *xy) {
     if (!b || !xy) return PF_ERR_ARG;
     Engine &e = b->e;
-    pf_status s = engine_sync_status(e);
+    bool any = false;
+    for (int i = 0; i < e.n; ++i) any = any || engine_has_frame(e, i, frame_index);
+    const pf_status s = engine_sync_status(e, [&] {
+        if (!any) return cudaSuccess;
+        if (launch_gather_estimates(e.d_trk, e.n, frame_index, e.d_gather, e.stream) != 0) return cudaErrorLaunchFailure;
+        return cudaMemcpyAsync(e.h_gather, e.d_gather, sizeof(double) * 2 * e.n, cudaMemcpyDeviceToHost, e.stream);
+    });
     if (s != PF_OK) return s;
     for (int i = 0; i < e.n; ++i) {
-        double v[2];
-        if (engine_read_frame(e, i, frame_index, v, nullptr) == PF_OK) {
-            xy[2 * i] = v[0];
-            xy[2 * i + 1] = v[1];
-        } else {
-            xy[2 * i] = NAN;
-            xy[2 * i + 1] = NAN;
-        }
+        const bool has = engine_has_frame(e, i, frame_index);
+        xy[2 * i] = has ? e.h_gather[2 * i] : NAN;
+        xy[2 * i + 1] = has ? e.h_gather[2 * i + 1] : NAN;
     }
-    return e.sticky;
+    return PF_OK;
 }
 
 pf_status pf_batch_destroy(pf_batch *b) {

@@ -145,7 +145,7 @@ struct LaunchItem {
 };
 
 struct LaunchRec {
-    int32_t *h_pos = nullptr, *d_pos = nullptr;         // slot_of[cap] then tile_prefix[cap + 1]
+    // one block copied in one piece: frames[n], then slot_of[n], then tile_prefix[n + 1]
     FrameRef *h_frames = nullptr, *d_frames = nullptr;
     double *h_est = nullptr, *d_est = nullptr;
     std::vector<LaunchItem> items;
@@ -164,6 +164,7 @@ struct Engine {
     std::vector<LaunchRec *> recs;
     int next = 0;
     std::vector<int> free_slots;
+    TrackerState *h_states = nullptr;   // pinned copy of d_states (status words of a drained server)
 };
 
 void CUDART_CB launch_done(void *p) {
@@ -193,6 +194,9 @@ struct pf_server {
 
 namespace {
 
+// Bytes of a launch's block for n streams: their frame references, slots and tile prefix.
+size_t launch_block_bytes(int n) { return sizeof(FrameRef) * n + sizeof(int32_t) * (2 * static_cast<size_t>(n) + 1); }
+
 pf_status engine_init(pf_server *S, int prec) {
     Engine &e = S->eng[prec];
     if (e.prec >= 0) return PF_OK;
@@ -203,14 +207,14 @@ pf_status engine_init(pf_server *S, int prec) {
     if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&e.d_states), sizeof(TrackerState) * cap);
     if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&e.d_ticket), sizeof(uint32_t));
     if (err == cudaSuccess) err = cudaMemsetAsync(e.d_ticket, 0, sizeof(uint32_t), e.stream);
+    if (err == cudaSuccess) err = cudaMallocHost(reinterpret_cast<void **>(&e.h_states), sizeof(TrackerState) * cap);
+    const size_t block = launch_block_bytes(cap);
     for (int k = 0; err == cudaSuccess && k < S->cfg.max_in_flight; ++k) {
         LaunchRec *r = new (std::nothrow) LaunchRec();
         if (!r) { err = cudaErrorMemoryAllocation; break; }
         e.recs.push_back(r);
-        err = cudaMallocHost(reinterpret_cast<void **>(&r->h_pos), sizeof(int32_t) * (2 * cap + 1));
-        if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&r->d_pos), sizeof(int32_t) * (2 * cap + 1));
-        if (err == cudaSuccess) err = cudaMallocHost(reinterpret_cast<void **>(&r->h_frames), sizeof(FrameRef) * cap);
-        if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&r->d_frames), sizeof(FrameRef) * cap);
+        err = cudaMallocHost(reinterpret_cast<void **>(&r->h_frames), block);
+        if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&r->d_frames), block);
         if (err == cudaSuccess) err = cudaMallocHost(reinterpret_cast<void **>(&r->h_est), sizeof(double) * 2 * cap);
         if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&r->d_est), sizeof(double) * 2 * cap);
     }
@@ -227,12 +231,12 @@ pf_status engine_init(pf_server *S, int prec) {
 void engine_free(Engine &e) {
     if (e.stream) cudaStreamSynchronize(e.stream);
     for (LaunchRec *r : e.recs) {
-        cudaFreeHost(r->h_pos); cudaFree(r->d_pos);
         cudaFreeHost(r->h_frames); cudaFree(r->d_frames);
         cudaFreeHost(r->h_est); cudaFree(r->d_est);
         delete r;
     }
     e.recs.clear();
+    if (e.h_states) cudaFreeHost(e.h_states);
     cudaFree(e.d_trk); cudaFree(e.d_states); cudaFree(e.d_ticket);
     if (e.stream) cudaStreamDestroy(e.stream);
     e = Engine();
@@ -286,8 +290,6 @@ pf_status launch_engine(pf_server *S, Engine &e, int *launched) {
         if (!st.open || st.cfg.precision != e.prec || st.queued.empty()) continue;
         const Pending pd = st.queued.front();
         st.queued.pop_front();
-        r->h_pos[n] = st.slot;
-        r->h_pos[cap + n] = tiles;
         FrameRef fr;
         memset(&fr, 0, sizeof fr);
         fr.base = pd.frame;
@@ -298,24 +300,28 @@ pf_status launch_engine(pf_server *S, Engine &e, int *launched) {
         if (pd.ring_slot >= 0 && err == cudaSuccess) err = cudaStreamWaitEvent(e.stream, st.ring_ev[pd.ring_slot], 0);
         r->items.push_back(LaunchItem{sid, pd.index, pd.arrival, pd.ring_slot});
         st.in_flight++;
-        tiles += st.lay.ntiles;
         ++n;
     }
     if (n == 0) return PF_OK;
-    r->h_pos[cap + n] = tiles;
-    // slot_of at d_pos[0..n), tile prefix at d_pos[cap .. cap + n]
-    if (err == cudaSuccess) err = cudaMemcpyAsync(r->d_pos, r->h_pos, sizeof(int32_t) * n, cudaMemcpyHostToDevice, e.stream);
+    int32_t *h_slot = reinterpret_cast<int32_t *>(r->h_frames + n), *h_prefix = h_slot + n;
+    for (int k = 0; k < n; ++k) {
+        const Stream &st = S->streams[r->items[k].stream];
+        h_slot[k] = st.slot;
+        h_prefix[k] = tiles;
+        tiles += st.lay.ntiles;
+    }
+    h_prefix[n] = tiles;
     if (err == cudaSuccess)
-        err = cudaMemcpyAsync(r->d_pos + cap, r->h_pos + cap, sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, e.stream);
-    if (err == cudaSuccess) err = cudaMemcpyAsync(r->d_frames, r->h_frames, sizeof(FrameRef) * n, cudaMemcpyHostToDevice, e.stream);
+        err = cudaMemcpyAsync(r->d_frames, r->h_frames, launch_block_bytes(n), cudaMemcpyHostToDevice, e.stream);
     if (err != cudaSuccess) { cudaGetLastError(); return S->fail(PF_ERR_CUDA); }
+    const int32_t *d_slot = reinterpret_cast<const int32_t *>(r->d_frames + n);
     StepLaunch L;
     L.trk = e.d_trk;
     L.states = e.d_states;
     L.frames = r->d_frames;
     L.tile_trk = nullptr;
-    L.tile_prefix = r->d_pos + cap;
-    L.slot_of = r->d_pos;
+    L.tile_prefix = d_slot + n;
+    L.slot_of = d_slot;
     L.est_out = r->d_est;
     L.ticket = e.d_ticket;
     L.ntrk = n;
@@ -339,13 +345,14 @@ pf_status launch_engine(pf_server *S, Engine &e, int *launched) {
 pf_status check_status(pf_server *S) {
     for (Engine &e : S->eng) {
         if (e.prec < 0) continue;
+        // every slot's state in one copy (a blocking copy per stream cost 8 us each)
+        cudaError_t err = cudaMemcpyAsync(e.h_states, e.d_states, sizeof(TrackerState) * S->cfg.max_streams,
+                                          cudaMemcpyDeviceToHost, e.stream);
+        if (err == cudaSuccess) err = cudaStreamSynchronize(e.stream);
+        if (err != cudaSuccess) { cudaGetLastError(); return S->fail(PF_ERR_CUDA); }
         for (const Stream &st : S->streams) {
             if (!st.open || st.cfg.precision != e.prec) continue;
-            uint32_t status = 0;
-            if (cudaMemcpy(&status, &e.d_states[st.slot].status, sizeof status, cudaMemcpyDeviceToHost) != cudaSuccess) {
-                cudaGetLastError();
-                return S->fail(PF_ERR_CUDA);
-            }
+            const uint32_t status = e.h_states[st.slot].status;
             if (status & kStatusTimeout) return S->fail(PF_ERR_TIMEOUT);
             if (status & kStatusBounds) return S->fail(PF_ERR_STATE);   // checked builds
         }
