@@ -797,40 +797,12 @@ __device__ __forceinline__ int upper_index(const int32_t *J, int n, int j) {
     return lo;
 }
 
-// Merge of the tracker's tile partials (one per thread, all loads in flight, then the
-// block merge: deterministic) and the new state, by the tile that completed the tracker.
-template <int P>
-__device__ void finalize_tracker(const TrackerDev &T, TrackerState *st, StepSmem<P> &sm, double *est_out,
-                                 bool track_box) {
-    using acc_t = typename Prec<P>::acc_t;
+// The new state from a tracker's merged statistics (in every lane of the first warp).
+template <int P, typename A>
+__device__ __forceinline__ void finish_tracker(const TrackerDev &T, TrackerState *st, StepSmem<P> &sm, Stats<A> v,
+                                               float4 bb, double *est_out, bool track_box) {
+    using acc_t = A;
     constexpr bool kF64 = sizeof(acc_t) == 8;
-    constexpr bool F = Prec<P>::kHalf;
-    Stats<acc_t> v{neg_inf<acc_t>(), 0, 0, 0};
-    float4 bb = make_float4(FLT_MAX, -FLT_MAX, FLT_MAX, -FLT_MAX);
-    const uint64_t tg = partial_tag(sm.st.epoch);
-    for (int i = threadIdx.x; i < T.ntiles; i += kThreads) {
-        Stats<acc_t> w;
-        uint64_t q[8];
-        if constexpr (kF64) {
-            const double *p = T.part[i].d;
-            w = Stats<acc_t>{__ldcg(p + 0), __ldcg(p + 1), __ldcg(p + 2), __ldcg(p + 3)};
-            const unsigned long long *pb = reinterpret_cast<const unsigned long long *>(T.part[i].b);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) q[4 + k] = track_box ? __ldcg(pb + k) : 0ull;
-        } else {
-            wait_partial(&T.part[i], tg, st, q, track_box);
-            w = Stats<acc_t>{__uint_as_float(static_cast<uint32_t>(q[0])), __uint_as_float(static_cast<uint32_t>(q[1])),
-                             __uint_as_float(static_cast<uint32_t>(q[2])), __uint_as_float(static_cast<uint32_t>(q[3]))};
-        }
-        v = stats_merge<F>(v, w);
-        bb.x = fminf(bb.x, __uint_as_float(static_cast<uint32_t>(q[4])));
-        bb.y = fmaxf(bb.y, __uint_as_float(static_cast<uint32_t>(q[5])));
-        bb.z = fminf(bb.z, __uint_as_float(static_cast<uint32_t>(q[6])));
-        bb.w = fmaxf(bb.w, __uint_as_float(static_cast<uint32_t>(q[7])));
-    }
-    if (track_box) warp_box(bb, sm);
-    v = block_stats<P>(v, sm);
-    if (track_box && threadIdx.x < 32) bb = merge_warp_boxes(sm);
     if (threadIdx.x < 32) {
         // The new state, from the block's statistics (thread 0's, broadcast) and this launch's
         // starting state (the copy in shared memory, which no tile changes), written field by
@@ -897,6 +869,44 @@ __device__ void finalize_tracker(const TrackerDev &T, TrackerState *st, StepSmem
             *T.done = 0u;
         }
     }
+}
+
+// The tile that completed the tracker: all partials merged (one per thread, all loads in
+// flight, then the block merge: deterministic), then the new state.
+template <int P>
+__device__ void finalize_tracker(const TrackerDev &T, TrackerState *st, StepSmem<P> &sm, double *est_out,
+                                 bool track_box) {
+    using acc_t = typename Prec<P>::acc_t;
+    constexpr bool kF64 = sizeof(acc_t) == 8;
+    constexpr bool F = Prec<P>::kHalf;
+    Stats<acc_t> v{neg_inf<acc_t>(), 0, 0, 0};
+    float4 bb = make_float4(FLT_MAX, -FLT_MAX, FLT_MAX, -FLT_MAX);
+    const uint64_t tg = partial_tag(sm.st.epoch);
+    for (int i = threadIdx.x; i < T.ntiles; i += kThreads) {
+        Stats<acc_t> w;
+        uint64_t q[8];
+        if constexpr (kF64) {
+            const double *p = T.part[i].d;
+            w = Stats<acc_t>{__ldcg(p + 0), __ldcg(p + 1), __ldcg(p + 2), __ldcg(p + 3)};
+            const unsigned long long *pb = reinterpret_cast<const unsigned long long *>(T.part[i].b);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) q[4 + k] = track_box ? __ldcg(pb + k) : 0ull;
+        } else {
+            wait_partial(&T.part[i], tg, st, q, track_box);
+            w = Stats<acc_t>{__uint_as_float(static_cast<uint32_t>(q[0])), __uint_as_float(static_cast<uint32_t>(q[1])),
+                             __uint_as_float(static_cast<uint32_t>(q[2])), __uint_as_float(static_cast<uint32_t>(q[3]))};
+        }
+        v = stats_merge<F>(v, w);
+        bb.x = fminf(bb.x, __uint_as_float(static_cast<uint32_t>(q[4])));
+        bb.y = fmaxf(bb.y, __uint_as_float(static_cast<uint32_t>(q[5])));
+        bb.z = fminf(bb.z, __uint_as_float(static_cast<uint32_t>(q[6])));
+        bb.w = fmaxf(bb.w, __uint_as_float(static_cast<uint32_t>(q[7])));
+    }
+    __syncthreads();              // (sm.red and sm.box still hold the tile's own)
+    if (track_box) warp_box(bb, sm);
+    v = block_stats<P>(v, sm);
+    if (track_box && threadIdx.x < 32) bb = merge_warp_boxes(sm);
+    finish_tracker<P>(T, st, sm, v, bb, est_out, track_box);
 }
 
 // The tracker's likelihood table of this launch into the tile's shared-memory table: each
@@ -1300,6 +1310,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             if (lane >= o) x += y;
         }
         if (lane == 31) sm.warp_sum[warp] = x;
+        if (kMode != kModeCdf && !gt) warp_box(make_float4(bx0, bx1, by0, by1), sm);   // (merged after the barrier)
         acc_t xex = __shfl_up_sync(0xffffffffu, x, 1);
         if (lane == 0) xex = static_cast<acc_t>(0);
         __syncthreads();
@@ -1440,7 +1451,10 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
     // lookback, so that the predecessors publish meanwhile.  (The pull kernel sizes it by
     // the gathered ancestors; the CDF kernel has none.)
     if constexpr (kMode != kModeCdf) {
-        if (!gt) warp_box(make_float4(bx0, bx1, by0, by1), sm);   // warp 0 merges them after the barrier
+        if (!gt && (kPull || t == 0)) {   // (else the scan's barrier ordered the warps' boxes)
+            warp_box(make_float4(bx0, bx1, by0, by1), sm);
+            __syncthreads();
+        }
         // the tracker table's share of this tile (after the aggregate is out)
         if (gt) {
             const uint64_t gtag = static_cast<uint64_t>(sm.st.epoch % 0x7fffffffu + 1u) << 32;
@@ -1466,7 +1480,6 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             sm.skeys[0] = T.key_lo; sm.skeys[1] = T.key_hi;
             sm.skeys[2] = static_cast<uint32_t>(t - 1); sm.skeys[3] = T.tracker_id;
         }
-        __syncthreads();
         if (!gt && warp == 0) {   // the block's box, in every lane of warp 0
             const float4 b = merge_warp_boxes(sm);
             bx0 = b.x; bx1 = b.y; by0 = b.z; by1 = b.w;
@@ -1498,7 +1511,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             }
             sm.win_x0 = x0; sm.win_y0 = y0; sm.win_w = ww; sm.win_h = wh;
         }
-        if (!gt) __syncthreads();
+        __syncthreads();
     }
     const bool no_table = kMode == kModeCdf;
     const int wx0 = no_table ? 0 : sm.win_x0, wy0 = no_table ? 0 : sm.win_y0;
@@ -2013,6 +2026,11 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
     if (track_box) warp_box(bb, sm);
     const Stats<acc_t> tot = block_stats<P>(stats, sm);
     if (track_box && warp == 0) bb = merge_warp_boxes(sm);
+    double *const est_out = Lp.est_out ? Lp.est_out + 2 * ti : nullptr;
+    if (T.ntiles == 1) {   // its statistics are the tracker's: no partial, no wait
+        finish_tracker<P>(T, st, sm, tot, bb, est_out, track_box);
+        return;
+    }
     if (tid == 0) {
         TilePartial *p = &T.part[PF_IDX(lt, T.ntiles)];
         if (track_box) {
@@ -2020,27 +2038,28 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             st_relaxed_v2(&p->b[0], btg | __float_as_uint(bb.x), btg | __float_as_uint(bb.y));
             st_relaxed_v2(&p->b[2], btg | __float_as_uint(bb.z), btg | __float_as_uint(bb.w));
         }
-        uint32_t prev;
         if constexpr (kF64) {
             p->d[0] = tot.m;
             p->d[1] = tot.s;
             p->d[2] = tot.sx;
             p->d[3] = tot.sy;
             // release: the partial is visible before the count; acquire: the last tile sees all
-            prev = atom_add_acq_rel(T.done, 1u);
+            sm.last = atom_add_acq_rel(T.done, 1u) == static_cast<uint32_t>(T.ntiles - 1) ? 1u : 0u;
         } else {
             const uint64_t tg = partial_tag(sm.st.epoch);
             st_relaxed_v2(&p->w[0], tg | __float_as_uint(tot.m), tg | __float_as_uint(tot.s));
             st_relaxed_v2(&p->w[2], tg | __float_as_uint(tot.sx), tg | __float_as_uint(tot.sy));
-            // the tracker's last tile finalises, waiting for every partial's tag: no tile waits
-            // for a counter's round trip (the tiles before it hold lower tickets, so they are
-            // running or done)
-            prev = static_cast<uint32_t>(lt);
         }
-        sm.last = (prev == static_cast<uint32_t>(T.ntiles - 1)) ? 1u : 0u;
     }
-    __syncthreads();
-    if (sm.last) finalize_tracker<P>(T, st, sm, Lp.est_out ? Lp.est_out + 2 * ti : nullptr, track_box);
+    // The tracker's last tile finalises, waiting for every partial's tag: no tile waits for a
+    // counter's round trip (the tiles before it hold lower tickets, so they are running or
+    // done).  REF64, whose partials carry no tags: the last tile to arrive.
+    bool last = lt == T.ntiles - 1;
+    if constexpr (kF64) {
+        __syncthreads();
+        last = sm.last != 0u;
+    }
+    if (last) finalize_tracker<P>(T, st, sm, est_out, track_box);
 }
 
 // CTAs per SM the register allocation must allow: 1024 threads per SM (64 registers a
