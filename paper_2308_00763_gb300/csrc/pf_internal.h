@@ -144,6 +144,7 @@ struct TrackerDev {
     void *dbg_cdf;
     int32_t *dbg_win;          // NULL unless PF_FLAG_DEBUG_ARRAYS: each tile's table window [4 * ntiles]
     void *cdf;                 // multinomial: the normalised CDF of the previous frame [N] (FP64 / FP32)
+    void *cdf8, *cdf64;        // ... and its values at the end of every 8 and 64 entries
     int32_t *anc;              // Gumbel-max, Metropolis, rejection: the ancestor of every offspring [N]
     LookbackDesc *look;
     TilePartial *part;

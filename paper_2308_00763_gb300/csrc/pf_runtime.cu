@@ -207,7 +207,7 @@ static pf_status engine_init(Engine &e, const pf_config *cfgs, int n, void *stre
     const size_t pb = pos_bytes(e.prec);
     const size_t cdf_b = e.prec == PF_REF64 ? 8 : 4;
     Arena a;
-    struct Off { size_t px[2], py[2], pl[2], look, part, done, state, est, stat, dbga, dbgc, dbgw, cdf, gtab; };
+    struct Off { size_t px[2], py[2], pl[2], look, part, done, state, est, stat, dbga, dbgc, dbgw, cdf, cdf8, cdf64, gtab; };
     std::vector<Off> off(n);
     // the trackers' states form one array (the kernel indexes it by tracker)
     const size_t states_off = a.take(sizeof(TrackerState) * n);
@@ -252,7 +252,11 @@ static pf_status engine_init(Engine &e, const pf_config *cfgs, int n, void *stre
             if (!multi) o.dbgc = a.take(cdf_b * N);
             o.dbgw = a.take(sizeof(int32_t) * 4 * static_cast<size_t>(nt));
         }
-        if (multi) o.cdf = a.take((given ? sizeof(int32_t) : cdf_b) * N + 16);
+        if (multi) o.cdf = a.take((given ? sizeof(int32_t) : cdf_b) * N + 64);
+        if (multi && !given) {   // whole groups of 8 are read: room up to a multiple of 64 entries
+            o.cdf8 = a.take(cdf_b * 8 * ((N + 63) / 64));
+            o.cdf64 = a.take(cdf_b * ((N + 63) / 64));
+        }
         if (given) {
             const int s = c.resampler == PF_RESAMPLE_GUMBEL ? 0 : c.resampler == PF_RESAMPLE_METROPOLIS ? 1 : 2;
             const int per = s == 0 ? kGumbelOffspring : s == 1 ? kMetropolisThreads : kRejectionOffspring;
@@ -330,6 +334,8 @@ static pf_status engine_init(Engine &e, const pf_config *cfgs, int n, void *stre
         if (e.cfg[i].resampler == PF_RESAMPLE_MULTINOMIAL) {
             // written by the CDF kernel, read by the pull kernel and by pf_get_debug
             T.cdf = e.d_arena + o.cdf;
+            T.cdf8 = e.d_arena + o.cdf8;
+            T.cdf64 = e.d_arena + o.cdf64;
             T.dbg_cdf = T.cdf;
         }
         if (ancestors_given(e.cfg[i].resampler)) {
