@@ -231,7 +231,7 @@ int step_grid_size(int precision, int total_tiles);
 // of full tiles (SMs x CTAs per SM x kTile / 2 particles) takes the smallest multiple of
 // 8 that splits it into a whole number of waves of the device's resident CTAs, so every
 // tile carries the same load (between kTile / 2 and kTile); a smaller tracker takes
-// kTile.  A function of (precision, n, device model) only, so a tracker tiles the same
+// kTile (REF64: one tile an SM, of at least 1024 particles).  A function of (precision, n, device model) only, so a tracker tiles the same
 // alone, in a batch and through the allocation-free entry point.
 int step_tile_size(int precision, int64_t n);
 int launch_debug_philox(const uint32_t *d_ctrs, int64_t n, uint64_t seed, uint32_t *d_out,
