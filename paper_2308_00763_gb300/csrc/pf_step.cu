@@ -383,6 +383,15 @@ __device__ __forceinline__ void store_items(T *dst, const T (&src)[kItems]) {
 
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
+// t mod n for t >= 0 and 0 < n <= 2^16, in 32-bit divisions: a 64-bit one is a called routine, around
+// which registers of the whole tile were spilled (F16 2^20 particles 20.0 -> 19.6 us a frame).
+__device__ __forceinline__ int64_t mod_small(int64_t t, uint32_t n) {
+    const uint32_t hi = static_cast<uint32_t>(static_cast<uint64_t>(t) >> 32), lo = static_cast<uint32_t>(t);
+    uint32_t r = hi % n;
+    r = ((r << 16) | (lo >> 16)) % n;
+    return ((r << 16) | (lo & 0xffffu)) % n;
+}
+
 struct FrameView {
     const uint8_t *p;
     int64_t pitch;
@@ -1269,7 +1278,8 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
     fv.W = T.W; fv.H = T.H; fv.r = T.r;
     if (Lp.frame_override) { fv.p = Lp.frame_override; fv.pitch = Lp.pitch_override; }
     else {
-        const int64_t ft = sm.fr.ring ? t % sm.fr.ring : t;   // a ring of staged frames, or a resident video
+        // a ring of staged frames, or a resident video
+        const int64_t ft = sm.fr.ring ? mod_small(t, static_cast<uint32_t>(sm.fr.ring)) : t;
         fv.p = sm.fr.base + (sm.fr.stride ? ft * sm.fr.stride : 0);
         fv.pitch = sm.fr.pitch;
     }
