@@ -680,6 +680,7 @@ struct __align__(16) StepSmem {
     int jbeg, jend;           // the tile's offspring are j in [jbeg, jend)
     double u0d;               // resampling offset u0 of the previous frame
     float u0f;
+    alignas(16) uint32_t rk[20];   // Philox round keys of the tracker
     uint32_t skeys[4];        // stratified resampling: key_lo, key_hi, frame t - 1, tracker id
     int win_x0, win_y0, win_w, win_h;   // likelihood table window (win_w = 0: none)
     int qmin;
@@ -1521,6 +1522,9 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
                 if (lane == 0) st_relaxed_u64(&T.gtab[PF_IDX(c, kTableMax)], gtag | payload);
             }
         }
+        if (tid >= 64 && tid < 84)   // the round keys of the propagation draws (ordered by the barrier below)
+            sm.rk[tid - 64] = (tid & 1) ? T.key_hi + static_cast<uint32_t>((tid - 64) >> 1) * 0xBB67AE85u
+                                        : T.key_lo + static_cast<uint32_t>((tid - 64) >> 1) * 0x9E3779B9u;
         // the resampling offset u0 of frame t - 1 (Philox tag 1, index 0), once per tile
         if (t > 0 && tid == 32) {
             const uint32_t w0 =
@@ -1868,7 +1872,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
     lik_t *__restrict__ Lout = static_cast<lik_t *>(T.pl[out]);
     int32_t *__restrict__ dbg_anc = T.dbg_anc;
     const uint32_t tctr = static_cast<uint32_t>(t);
-    const uint32_t trk_id = T.tracker_id, key_lo = T.key_lo, key_hi = T.key_hi;
+    const uint32_t trk_id = T.tracker_id;
     const int jpair0 = static_cast<int>(T.j_base >> 1);   // global pair index of local pair 0
     Stats<acc_t> stats{neg_inf<acc_t>(), 0, 0, 0};
     const acc_t nxa_a = static_cast<acc_t>(nxi), nya_a = static_cast<acc_t>(nyi);
@@ -1932,7 +1936,8 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
         }
         // one Philox block per particle pair: words (x, y) for j0, (z, w) for j1 (a shard's
         // pairs are numbered globally)
-        const uint4 wd = philox4x32_10(make_uint4(static_cast<uint32_t>(q + jpair0), tctr, 0u, trk_id), key_lo, key_hi);
+        const uint4 wd = philox4x32_10_keys(make_uint4(static_cast<uint32_t>(q + jpair0), tctr, 0u, trk_id),
+                                            reinterpret_cast<const uint4 *>(sm.rk));
 
         if constexpr (!Tr::kHalf) {
             // ---------------- REF64 / F32: absolute positions, exact-integer likelihood
