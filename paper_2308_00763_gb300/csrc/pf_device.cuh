@@ -44,6 +44,11 @@ __device__ __forceinline__ uint4 philox4x32_10_keys(uint4 c, const uint4 *rk) {
     return c;
 }
 
+// Round key word i (0 <= i < 20) of philox4x32_10_keys.
+__device__ __forceinline__ uint32_t philox_round_key(int i, uint32_t key_lo, uint32_t key_hi) {
+    return (i & 1) ? key_hi + static_cast<uint32_t>(i >> 1) * 0xBB67AE85u : key_lo + static_cast<uint32_t>(i >> 1) * 0x9E3779B9u;
+}
+
 // Uniform on (0,1) from the top 23 bits: ((w >> 9) + 1/2) * 2^-23, exact in FP32 and FP64, so
 // every precision sees the same uniforms.  One funnel shift puts the 23 bits under the
 // exponent of [1, 2) and one exact addition takes 1 - 2^-24 off: no integer-to-float

@@ -30,7 +30,8 @@
 // warp shuffles, then one thread per offspring over the warps' results.  The pull kernel
 // gathers the ancestors written here.
 // Measured us a frame on the tracker's peaked weights, every variate in full -> these tests: F32
-// 8191 particles 166 -> 108, REF64 2047 543 -> 254.
+// 8191 particles 166 -> 106, REF64 2047 543 -> 247; with the round keys in shared memory and wide
+// products in the generator F32 86.
 #include <math.h>
 
 #include "pf_ancestor.cuh"
@@ -62,6 +63,7 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
     __shared__ int s_k[kWarps][kJ];
     __shared__ uint16_t s_list[kGumbelMaxN / 4];   // quads with a particle that can win
     __shared__ unsigned int s_n;
+    __shared__ alignas(16) uint32_t s_rk[20];      // Philox round keys
     __shared__ acc_t s_max[kWarps];
     __shared__ unsigned int s_eb[kJ];              // exp(best - max L) of the CTA, float bits (>= 0)
 
@@ -76,7 +78,7 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
     const int j0 = (b - __ldg(G.cta_prefix + g)) * kJ;
     const lik_t *__restrict__ L = static_cast<const lik_t *>(T.pl[static_cast<int>((t + 1) & 1)]);
     const uint32_t tctr = static_cast<uint32_t>(t - 1);
-    const uint32_t key_lo = T.key_lo, key_hi = T.key_hi, trk_id = T.tracker_id;
+    const uint32_t trk_id = T.tracker_id;
 
     acc_t best[kJ];
     int arg[kJ];
@@ -100,6 +102,8 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
     }
     if (lane == 0) s_max[wid] = mx;
     if (threadIdx.x == 0) s_n = 0u;
+    if (threadIdx.x < 20) s_rk[threadIdx.x] = philox_round_key(threadIdx.x, T.key_lo, T.key_hi);
+    const uint4 *rk = reinterpret_cast<const uint4 *>(s_rk);
     if (threadIdx.x < kJ) s_eb[threadIdx.x] = 0u;
     __syncthreads();
 #pragma unroll
@@ -136,9 +140,9 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
         for (int jj = 0; jj < kJ; ++jj) {
             const int j = j0 + jj;
             if (j >= N) break;
-            const uint4 w = philox4x32_10(make_uint4(static_cast<uint32_t>(q), tctr, 4u + (static_cast<uint32_t>(j) << 8),
+            const uint4 w = philox4x32_10_keys(make_uint4(static_cast<uint32_t>(q), tctr, 4u + (static_cast<uint32_t>(j) << 8),
                                                      trk_id),
-                                          key_lo, key_hi);
+                                          rk);
             const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
             const float eb = __uint_as_float(*reinterpret_cast<volatile unsigned int *>(&s_eb[jj]));
 #pragma unroll

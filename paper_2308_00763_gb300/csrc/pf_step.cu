@@ -1542,8 +1542,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             }
         }
         if (tid >= 64 && tid < 84)   // the round keys of the propagation draws (ordered by the barrier below)
-            sm.rk[tid - 64] = (tid & 1) ? T.key_hi + static_cast<uint32_t>((tid - 64) >> 1) * 0xBB67AE85u
-                                        : T.key_lo + static_cast<uint32_t>((tid - 64) >> 1) * 0x9E3779B9u;
+            sm.rk[tid - 64] = philox_round_key(tid - 64, T.key_lo, T.key_hi);
         // the resampling offset u0 of frame t - 1 (Philox tag 1, index 0), once per tile
         if (t > 0 && tid == 32) {
             const uint32_t w0 =
