@@ -1,7 +1,8 @@
 // pf_step.cu -- the fused per-frame SIR step for sm_103a.
 //
 // One launch per frame for a whole batch of trackers.  A tile is kTile consecutive
-// particles k of one tracker's previous frame.  Per tile (dynamic ticket order):
+// particles k of one tracker's previous frame.  Per tile (in ticket order; a CTA's first ticket
+// is its index):
 //   1. resampling of the previous frame (Sec. IV, "Normalizing" and "Resampling"):
 //      e_k = exp(L_k - M) (Eq. 5 with the max of the previous step), a block scan, and a
 //      decoupled lookback over the tracker's earlier tiles give the inclusive prefix
@@ -28,7 +29,7 @@
 // the weights) are not in the step kernel's launch; they take two other launches per
 // frame (the same code in other modes): the CDF kernel runs phase 1 up to the CDF and writes it to
 // T.cdf; the pull kernel then gives each offspring j the first particle whose CDF value
-// reaches an independent uniform v_j (a binary search over T.cdf), gathers the ancestors'
+// reaches an independent uniform v_j (a search of T.cdf in three levels), gathers the ancestors'
 // positions of its tile's offspring into shared memory, sizes the likelihood window by
 // them and runs phases 2-5 as the step kernel does.  Gumbel-max trackers (the log-domain
 // form of the same draw, Sec. IV), Metropolis and rejection trackers (Sec. III) skip the CDF
@@ -1165,8 +1166,7 @@ __device__ __forceinline__ void table_by_rows(StepSmem<P> &sm, int rw, int pw, i
 // found, read as whole sectors and counted; the eight entries below that, likewise.  The chain
 // of dependent reads from L2 is two long, where a bisection below a coarse table took seven or
 // eight, most of them a sector each.  C is non-decreasing and its last value is 1, so the index
-// is that of a search of the whole CDF.  Measured us a frame: F16 2^19 particles 47.3 -> 41.1,
-// F32 300003 66.7 -> 43.8 (from the bisection's beginning).
+// is that of a search of the whole CDF.  Measured us a frame: F16 2^19 particles 47.3 -> 41.1.
 template <int P>
 __device__ __forceinline__ void cdf_search(const TrackerDev &T, const typename Prec<P>::acc_t (&u)[kItems], int (&k)[kItems],
                                            StepSmem<P> &sm, TrackerState *st) {
