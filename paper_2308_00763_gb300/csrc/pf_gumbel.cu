@@ -21,18 +21,24 @@
 //     logarithms, with a margin (1e-3 and 4e-6 max |L| relative) above the rounding of both sides.
 // Whoever passes is evaluated as before, so the argmax and its ties are the same.
 //
-// Layout: CTA b takes kGumbelOffspring consecutive offspring of one tracker.  Its threads
-// stride over the listed particle quads q (particles 4q .. 4q+3): one Philox block per (quad,
-// offspring) gives that offspring's four draws, the quad's four L are loaded once for all
-// of the CTA's offspring, and each thread keeps a running best per offspring (ties to the
-// smaller index).  The best of all threads, as exp(b_j - max L), is shared through shared
-// memory for the test above.  The CTA then reduces each offspring's (value, index) pairs:
-// warp shuffles, then one thread per offspring over the warps' results.  The pull kernel
-// gathers the ancestors written here.
-// Measured us a frame on the tracker's peaked weights, every variate in full -> these tests: F32
-// 8191 particles 166 -> 106, REF64 2047 543 -> 247; with the round keys in shared memory and wide
-// products in the generator F32 86.
+// Layout: CTA b takes kGumbelOffspring consecutive offspring of one tracker, thread i its
+// offspring i mod 8 over every 32nd listed particle quad q (particles 4q .. 4q+3), from quad i / 8
+// on: one Philox block per (quad, offspring) gives four draws, tested against the quad's four
+// exp(L_k - max L) in shared memory (computed once for the CTA's offspring, kGumbelChunk quads at
+// a time).  The best of an offspring's threads, as exp(b_j - max L), is shared through shared
+// memory for the test above; it starts at the bound that the particle of the largest L gives.
+// The CTA then reduces each offspring's (value, index) pairs, ties to the smaller index: two
+// shuffles, then one thread per offspring over the warps' results.  The pull kernel gathers the
+// ancestors written here.
+// (A thread that draws for all eight offspring of its quad meets the shared best only in its
+// second pass, after 1024 particles, leaves most threads idle on a short list, and holds 80
+// registers to this one's 46.)
+// Measured us a frame on the tracker's peaked weights, every variate in full -> these tests, a
+// thread for all eight offspring of a quad -> this layout: F32 8191 particles 170 -> 86 -> 53, F16
+// 1000 18.8 -> 21.4 -> 12.8, 2^16 10 040 -> 1144 -> 727, REF64 2047 603 -> 246 -> 103.
 #include <math.h>
+
+#include <type_traits>
 
 #include "pf_ancestor.cuh"
 #include "pf_device.cuh"
@@ -53,6 +59,28 @@ __device__ __forceinline__ void take_best(A &v, int &k, A v2, int k2) {
     }
 }
 
+constexpr int kGumbelChunk = 512;   // quads whose exp(L_k - max L) are in shared memory at a time
+static_assert(kGumbelOffspring <= 32 && 32 % kGumbelOffspring == 0, "a warp holds whole groups of the CTA's offspring");
+
+// The four L of particles k .. k + 3 (k a multiple of 4, L aligned to 16 bytes), -inf past the last.
+template <typename L_t, typename A>
+__device__ __forceinline__ void load_quad(const L_t *__restrict__ L, int k, int N, A (&l)[4]) {
+    if (k + 3 < N) {
+        using V = typename std::conditional<sizeof(L_t) == 2, uint2, uint4>::type;
+        union {
+            V v[4 * sizeof(L_t) / sizeof(V)];
+            L_t e[4];
+        } u;
+#pragma unroll
+        for (int i = 0; i < static_cast<int>(4 * sizeof(L_t) / sizeof(V)); ++i) u.v[i] = __ldg(reinterpret_cast<const V *>(L + k) + i);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) l[i] = to_acc(u.e[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) l[i] = k + i < N ? static_cast<A>(to_acc(L[k + i])) : static_cast<A>(-INFINITY);
+    }
+}
+
 template <int P>
 __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLaunch G) {
     using lik_t = typename Prec<P>::lik_t;
@@ -62,6 +90,7 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
     __shared__ acc_t s_v[kWarps][kJ];
     __shared__ int s_k[kWarps][kJ];
     __shared__ uint16_t s_list[kGumbelMaxN / 4];   // quads with a particle that can win
+    __shared__ float4 s_el[kGumbelChunk];          // margin * exp(L_k - max L) of a chunk of listed quads
     __shared__ unsigned int s_n;
     __shared__ alignas(16) uint32_t s_rk[20];      // Philox round keys
     __shared__ acc_t s_max[kWarps];
@@ -80,20 +109,15 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
     const uint32_t tctr = static_cast<uint32_t>(t - 1);
     const uint32_t trk_id = T.tracker_id;
 
-    acc_t best[kJ];
-    int arg[kJ];
-#pragma unroll
-    for (int jj = 0; jj < kJ; ++jj) {
-        best[jj] = -INFINITY;
-        arg[jj] = N;
-    }
     const int nq = (N + 3) >> 2;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     // the largest L (NaN aside) and the list of quads that can win
     acc_t mx = -INFINITY;
-    for (int k = threadIdx.x; k < N; k += kGumbelThreads) {
-        const acc_t l = to_acc(L[k]);
-        mx = l > mx ? l : mx;
+    for (int q = threadIdx.x; q < nq; q += kGumbelThreads) {
+        acc_t l[4];
+        load_quad(L, 4 * q, N, l);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) mx = l[i] > mx ? l[i] : mx;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -104,18 +128,22 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
     if (threadIdx.x == 0) s_n = 0u;
     if (threadIdx.x < 20) s_rk[threadIdx.x] = philox_round_key(threadIdx.x, T.key_lo, T.key_hi);
     const uint4 *rk = reinterpret_cast<const uint4 *>(s_rk);
-    if (threadIdx.x < kJ) s_eb[threadIdx.x] = 0u;
+    // exp(-2.82), rounded down: what the particle of the largest L is sure of
+    if (threadIdx.x < kJ) s_eb[threadIdx.x] = __float_as_uint(0.0595f);
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) mx = s_max[w] > mx ? s_max[w] : mx;
     const bool finite = mx - mx == static_cast<acc_t>(0);   // else every quad is evaluated in full
     const acc_t line = mx - static_cast<acc_t>(19.5) - static_cast<acc_t>(1e-5) * (mx < 0 ? -mx : mx);
     for (int q0 = 0; q0 < nq; q0 += kGumbelThreads) {
-        const int q = q0 + static_cast<int>(threadIdx.x), k = 4 * q;
+        const int q = q0 + static_cast<int>(threadIdx.x);
         bool keep = false;
         if (q < nq) {
+            acc_t l[4];
+            load_quad(L, 4 * q, N, l);
+            keep = !finite;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) keep = keep || (k + i < N && (!finite || to_acc(L[k + i]) >= line));
+            for (int i = 0; i < 4; ++i) keep = keep || l[i] >= line;
         }
         const uint32_t mask = __ballot_sync(0xffffffffu, keep);
         unsigned int at = 0;
@@ -127,19 +155,26 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
     const int nl = static_cast<int>(s_n);
     const float mxf = static_cast<float>(mx);
     const float margin = 1.001f + 4e-6f * fabsf(mxf);
-    for (int p = threadIdx.x; p < nl; p += kGumbelThreads) {
-        const int q = s_list[p], k = 4 * q;
-        acc_t l[4];
-        float el[4];
+    const int jj = threadIdx.x % kJ, j = j0 + jj;
+    acc_t best = -INFINITY;
+    int arg = N;
+    for (int c0 = 0; c0 < nl; c0 += kGumbelChunk) {
+        const int nc = nl - c0 < kGumbelChunk ? nl - c0 : kGumbelChunk;
+        if (c0 > 0) __syncthreads();
+        for (int p = threadIdx.x; p < nc; p += kGumbelThreads) {
+            acc_t l[4];
+            load_quad(L, 4 * static_cast<int>(s_list[c0 + p]), N, l);
+            float el[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            l[i] = (k + i < N) ? to_acc(L[k + i]) : static_cast<acc_t>(-INFINITY);
-            el[i] = margin * __expf(static_cast<float>(l[i] - mx));
+            for (int i = 0; i < 4; ++i) el[i] = margin * __expf(static_cast<float>(l[i] - mx));
+            s_el[p] = make_float4(el[0], el[1], el[2], el[3]);
         }
-#pragma unroll
-        for (int jj = 0; jj < kJ; ++jj) {
-            const int j = j0 + jj;
-            if (j >= N) break;
+        __syncthreads();
+        if (j >= N) continue;
+        for (int p = threadIdx.x / kJ; p < nc; p += kGumbelThreads / kJ) {
+            const int q = s_list[c0 + p], k = 4 * q;
+            const float4 e4 = s_el[p];
+            const float el[4] = {e4.x, e4.y, e4.z, e4.w};
             const uint4 w = philox4x32_10_keys(make_uint4(static_cast<uint32_t>(q), tctr, 4u + (static_cast<uint32_t>(j) << 8),
                                                      trk_id),
                                           rk);
@@ -150,10 +185,10 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
                 // (not taken when either side is NaN: evaluated in full)
                 if (finite && (1.0f - uniform_f32(ws[i])) * eb > el[i]) continue;
                 if (k + i < N) {
-                    const acc_t v = l[i] + gumbel_of(ws[i], acc_t{});
-                    if (v > best[jj] || (v == best[jj] && k + i < arg[jj] && arg[jj] < N)) {
-                        best[jj] = v;
-                        arg[jj] = k + i;
+                    const acc_t v = to_acc(L[k + i]) + gumbel_of(ws[i], acc_t{});
+                    if (v > best || (v == best && k + i < arg && arg < N)) {
+                        best = v;
+                        arg = k + i;
                         if (finite) atomicMax(&s_eb[jj], __float_as_uint(__expf(static_cast<float>(v - mx))));
                     }
                 }
@@ -161,23 +196,17 @@ __global__ void __launch_bounds__(kGumbelThreads) gumbel_kernel(const AncestorLa
         }
     }
 #pragma unroll
-    for (int jj = 0; jj < kJ; ++jj) {
-        acc_t v = best[jj];
-        int k = arg[jj];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const acc_t v2 = __shfl_xor_sync(0xffffffffu, v, o);
-            const int k2 = __shfl_xor_sync(0xffffffffu, k, o);
-            take_best(v, k, v2, k2);
-        }
-        if (lane == 0) {
-            s_v[wid][jj] = v;
-            s_k[wid][jj] = k;
-        }
+    for (int o = 16; o >= kJ; o >>= 1) {
+        const acc_t v2 = __shfl_xor_sync(0xffffffffu, best, o);
+        const int k2 = __shfl_xor_sync(0xffffffffu, arg, o);
+        take_best(best, arg, v2, k2);
+    }
+    if (lane < kJ) {
+        s_v[wid][lane] = best;
+        s_k[wid][lane] = arg;
     }
     __syncthreads();
     if (threadIdx.x < kJ) {
-        const int jj = threadIdx.x, j = j0 + jj;
         acc_t v = s_v[0][jj];
         int k = s_k[0][jj];
 #pragma unroll

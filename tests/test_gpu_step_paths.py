@@ -113,3 +113,22 @@ def test_gumbel_over_flat_weights(pf, prec):
     for j in bad:
         g = oracle.gumbel_variates(27, 0, int(j), n)
         assert abs(g[want[j]] - g[anc[j]]) <= (1e-12 if prec == "ref64" else 1e-5) * max(1.0, abs(like[0]))
+
+
+@pytest.mark.parametrize("n", [1, 2, 5, 33, 2047, 2049, 4101])
+def test_gumbel_list_chunks(pf, n):
+    """Flat weights list every quad, so n sets the list: a part of one quad, quads fewer than a
+    pass takes, and the edges of the 2048 particles whose weights are staged at a time."""
+    frames = np.full((2, 64, 64), 100, np.uint8)
+    f = pf.Filter(64, 64, n, 3, "f32", init=(32.0, 32.0), seed=29, flags=pf.PF_FLAG_DEBUG_ARRAYS, resampler="gumbel")
+    f.step(_cuda(frames)[0])
+    like = f.get_state()["L"].astype(np.float64)
+    f.step(_cuda(frames)[1])
+    anc = f.debug(0).astype(np.int64)
+    f.close()
+    want = oracle.resample_gumbel(like, 29, 0, 0, "f32")
+    bad = np.nonzero(anc != want)[0]   # (near ties of the two sides' logarithms)
+    assert bad.size <= 2
+    for j in bad:
+        g = oracle.gumbel_variates(29, 0, int(j), n)
+        assert abs(g[want[j]] - g[anc[j]]) <= 1e-5 * max(1.0, abs(like[0]))
