@@ -268,6 +268,35 @@ __device__ __forceinline__ Stats<A> stats_merge(const Stats<A> &a, const Stats<A
     return r;
 }
 
+// Order, equality with -inf and narrowing of FP64 values on their words: an FP64 comparison or
+// conversion takes as long as ten integer operations.  (-0 orders below +0; no NaN.)  The FP64
+// step issued 95 FP64 operations a particle, 21 of them comparisons and conversions; with these,
+// the pixel by integers, no exponential of the maximum itself and nothing issued by warps past
+// a tile's end: 200003 particles 70.0 -> 58.8 us a frame, 2^20 214 -> 190, 1000 43.6 -> 35.0,
+// the same bits.
+__device__ __forceinline__ long long order_key(double v) {
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ bool above(double a, double b) { return order_key(a) > order_key(b); }
+__device__ __forceinline__ bool above(float a, float b) { return a > b; }
+__device__ __forceinline__ bool is_neg_inf(double v) {
+    return static_cast<unsigned long long>(__double_as_longlong(v)) == 0xfff0000000000000ull;
+}
+__device__ __forceinline__ bool is_neg_inf(float v) { return v == neg_inf<float>(); }
+__device__ __forceinline__ float to_f32(float v) { return v; }
+__device__ __forceinline__ float to_f32(double v) {   // rounded to nearest, as the conversion does
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(v)), lo = static_cast<uint32_t>(__double2loint(v));
+    const uint32_t e = (hi >> 20) & 0x7ffu;
+    if (e < 897u || e > 1149u) return static_cast<float>(v);   // (zero, FP32 subnormal or beyond)
+    const uint32_t f = (hi & 0x80000000u) | ((((hi & 0x7fffffffu) - 0x38000000u) << 3) | (lo >> 29));
+    const uint32_t rem = lo & 0x1fffffffu;
+    return __uint_as_float(f + (rem > 0x10000000u || (rem == 0x10000000u && (f & 1u)) ? 1u : 0u));
+}
+// A weight above 2^-30 of the largest (weights are never negative).
+__device__ __forceinline__ bool counts_in_box(float w) { return w > 9.3132257461547852e-10f; }
+__device__ __forceinline__ bool counts_in_box(double w) { return __double_as_longlong(w) > 0x3e10000000000000ll; }
+
 // Two particles at once (a particle whose flag is false is skipped).  The rescale to a new
 // maximum is applied without a branch: when the maximum does not move the factor is
 // wexp(0) = 1 exactly (and 1 while no particle has been seen), so the sums are unchanged,
@@ -275,16 +304,33 @@ __device__ __forceinline__ Stats<A> stats_merge(const Stats<A> &a, const Stats<A
 template <bool F, typename A>
 __device__ __forceinline__ void stats_add2(Stats<A> &a, bool v0, A L0, A dx0, A dy0, bool v1, A L1, A dx1, A dy1) {
     const A l0 = v0 ? L0 : neg_inf<A>(), l1 = v1 ? L1 : neg_inf<A>();
-    const A mx = l0 > l1 ? l0 : l1;
-    const A nm = mx > a.m ? mx : a.m;
-    if (sizeof(A) == 4 || nm != a.m) {   // (a factor of 1 costs FP64 more than a branch)
+    A e0, e1;
+    if constexpr (sizeof(A) == 8) {
+        // FP64: a factor of 1 or a weight of 1 costs more than the branch around it
+        const bool first = above(l0, l1);
+        const A hi = first ? l0 : l1, lo = first ? l1 : l0;
+        if (above(hi, a.m)) {
+            if (!is_neg_inf(a.m)) {      // (the sums are 0 otherwise)
+                const A sc = wexp<F>(a.m - hi);
+                a.s = mul_rn(a.s, sc); a.sx = mul_rn(a.sx, sc); a.sy = mul_rn(a.sy, sc);
+            }
+            a.m = hi;
+        }
+        A eh = static_cast<A>(1), el = static_cast<A>(0);
+        if (above(a.m, hi)) eh = wexp<F>(hi - a.m);
+        if (v0 && v1) el = wexp<F>(lo - a.m);
+        e0 = v0 ? (first ? eh : el) : static_cast<A>(0);
+        e1 = v1 ? (first ? el : eh) : static_cast<A>(0);
+    } else {
+        const A mx = l0 > l1 ? l0 : l1;
+        const A nm = mx > a.m ? mx : a.m;
         const A sc = (nm == neg_inf<A>()) ? static_cast<A>(1)
                                           : ((a.m == neg_inf<A>()) ? static_cast<A>(0) : wexp<F>(a.m - nm));
         a.s = mul_rn(a.s, sc); a.sx = mul_rn(a.sx, sc); a.sy = mul_rn(a.sy, sc);
         a.m = nm;
+        e0 = v0 ? wexp<F>(l0 - a.m) : static_cast<A>(0);
+        e1 = v1 ? wexp<F>(l1 - a.m) : static_cast<A>(0);
     }
-    const A e0 = v0 ? wexp<F>(l0 - a.m) : static_cast<A>(0);
-    const A e1 = v1 ? wexp<F>(l1 - a.m) : static_cast<A>(0);
     // (rounded step by step: an exponential's own last operation is a multiplication, which must
     // not be fused with these)
     a.s = add_rn(a.s, add_rn(e0, e1));
@@ -306,19 +352,25 @@ __device__ __forceinline__ int pixel_of(double v) {
 
 // Column (or row) of a position's pixel in a window: pixel_of(v) - origin as an unsigned value,
 // and a value above any window's extent when the pixel lies outside [-2^20, 2^20] or v is not
-// finite (the caller then takes pixel_of).  floor(v + 1/2) is formed by adding 1.5 * 2^23
-// (FP32; 1.5 * 2^52 in FP64) rounded downwards, which leaves the integer in the low mantissa
-// bits: two additions and an integer subtraction instead of two clamps, an addition and a
-// conversion (a quarter-rate unit).  FP32 for |v| >= 2^22 and any other large or special v:
-// the sum's bits differ from those of 1.5 * 2^23 by at least 2^22 in either direction, which
-// stays outside the window after the subtraction (|origin| < 2^20); FP64: the high word tells.
+// finite (the caller then takes pixel_of).  FP32: floor(v + 1/2) is formed by adding 1.5 * 2^23
+// rounded downwards, which leaves the integer in the low mantissa bits: two additions and an
+// integer subtraction instead of two clamps, an addition and a conversion (a quarter-rate
+// unit).  For |v| >= 2^22 and any other large or special v the sum's bits differ from those of
+// 1.5 * 2^23 by at least 2^22 in either direction, which stays outside the window after the
+// subtraction (|origin| < 2^20).
 __device__ __forceinline__ unsigned window_offset(float v, int origin) {
     return __float_as_uint(__fadd_rd(__fadd_rn(v, 0.5f), 12582912.0f)) - (0x4B400000u + static_cast<unsigned>(origin));
 }
+// FP64: floor(v + 1/2) = (floor(2 v) + 1) >> 1 from the words, in integer operations.
 __device__ __forceinline__ unsigned window_offset(double v, int origin) {
-    const double t = __dadd_rd(__dadd_rn(v, 0.5), 6755399441055744.0);
-    const bool ok = static_cast<unsigned>(__double2hiint(t)) + 0xBCC80001u <= 1u;
-    return ok ? static_cast<unsigned>(__double2loint(t)) - static_cast<unsigned>(origin) : 0xffffffffu;
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(v)), lo = static_cast<uint32_t>(__double2loint(v));
+    const uint32_t m = (hi & 0xfffffu) | 0x100000u;
+    const int sh = 1042 - static_cast<int>((hi >> 20) & 0x7ffu);   // 2 |v| = (m + lo 2^-32) 2^-sh
+    const int s = sh < 31 ? sh : 31;                                // (m >> 31 = 0)
+    const uint32_t ip = m >> (s & 31);
+    const bool rest = (ip << (s & 31)) != m || lo != 0u;
+    const int fl = static_cast<int>(hi) < 0 ? -static_cast<int>(ip) - (rest ? 1 : 0) : static_cast<int>(ip);
+    return sh >= 0 ? static_cast<unsigned>((fl + 1) >> 1) - static_cast<unsigned>(origin) : 0xffffffffu;
 }
 
 // kItems consecutive elements between memory and registers as 16-byte vectors (kItems *
@@ -732,7 +784,7 @@ __device__ __forceinline__ double warp_max(double x) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const double y = __shfl_xor_sync(0xffffffffu, x, o);
-        x = y > x ? y : x;
+        x = above(y, x) ? y : x;
     }
     return x;
 }
@@ -741,8 +793,8 @@ template <int P, typename A>
 __device__ __forceinline__ Stats<A> warp_stats(Stats<A> v) {
     constexpr bool F = Prec<P>::kHalf;
     const A m = warp_max(v.m);
-    if (m == neg_inf<A>()) return Stats<A>{m, 0, 0, 0};
-    const A sc = (v.m == neg_inf<A>()) ? static_cast<A>(0) : wexp<F>(v.m - m);
+    if (is_neg_inf(m)) return Stats<A>{m, 0, 0, 0};
+    const A sc = is_neg_inf(v.m) ? static_cast<A>(0) : wexp<F>(v.m - m);
     A s = mul_rn(v.s, sc), sx = mul_rn(v.sx, sc), sy = mul_rn(v.sy, sc);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1400,25 +1452,35 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             reinterpret_cast<uint4 *>(sm.map)[tid + i * kThreads] = make_uint4(0u, 0u, 0u, 0u);
         const float sx = Tr::kHalf ? static_cast<float>(axi_anc) : 0.0f;
         const float sy = Tr::kHalf ? static_cast<float>(ayi_anc) : 0.0f;
+        // FP64: a warp wholly past the tile's end (a REF64 tile may hold a quarter of kTile)
+        // issues none of the arithmetic; its sums are 0, and no one reads its prefixes
+        const bool live = !kF64 || warp * 32 * kItems < cnt;
         acc_t run = static_cast<acc_t>(0);
+        if (!live) {
 #pragma unroll
-        for (int m = 0; m < kItems; ++m) {
-            const acc_t v = wexp<Tr::kHalf>(to_acc(lv[m]) - M);   // 0 past the tile's end
-            if (!gt && v > static_cast<acc_t>(9.3132257461547852e-10)) {   // weight above 2^-30 of the max
-                const float xa = static_cast<float>(to_acc(Bits<pos_t>::get(xr, m))) + sx;
-                const float ya = static_cast<float>(to_acc(Bits<pos_t>::get(yr, m))) + sy;
-                bx0 = fminf(bx0, xa); bx1 = fmaxf(bx1, xa);
-                by0 = fminf(by0, ya); by1 = fmaxf(by1, ya);
+            for (int m = 0; m < kItems; ++m) loc[m] = static_cast<acc_t>(0);
+        } else {
+#pragma unroll
+            for (int m = 0; m < kItems; ++m) {
+                const acc_t v = wexp<Tr::kHalf>(to_acc(lv[m]) - M);   // 0 past the tile's end
+                if (!gt && counts_in_box(v)) {
+                    const float xa = to_f32(to_acc(Bits<pos_t>::get(xr, m))) + sx;
+                    const float ya = to_f32(to_acc(Bits<pos_t>::get(yr, m))) + sy;
+                    bx0 = fminf(bx0, xa); bx1 = fmaxf(bx1, xa);
+                    by0 = fminf(by0, ya); by1 = fmaxf(by1, ya);
+                }
+                run = (m == 0) ? v : add_rn(run, v);
+                loc[m] = run;
             }
-            run = (m == 0) ? v : add_rn(run, v);
-            loc[m] = run;
         }
         // block exclusive scan of the thread totals
         acc_t x = run;
+        if (live) {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const acc_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
+            for (int o = 1; o < 32; o <<= 1) {
+                const acc_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
         }
         if (lane == 31) sm.warp_sum[warp] = x;
         if (kMode != kModeCdf && !gt) warp_box(make_float4(bx0, bx1, by0, by1), sm);   // (merged after the barrier)
@@ -1428,12 +1490,12 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
         acc_t wpre = static_cast<acc_t>(0);
 #pragma unroll
         for (int w = 0; w < kWarps; ++w) {
-            if (kF64 && w >= warp) break;      // (an FP64 addition not needed is not issued either)
+            if (kF64 && (w >= warp || !live)) break;   // (an FP64 addition not needed is not issued either)
             const acc_t v = sm.warp_sum[w];
             if (w < warp) wpre += v;
         }
         const acc_t off = wpre + xex;
-        if (tid != 0) {
+        if (tid != 0 && live) {
 #pragma unroll
             for (int m = 0; m < kItems; ++m) loc[m] = off + loc[m];
         }
@@ -1794,7 +1856,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
         const acc_t c_prev = prefix_min(PF_NORM(prefix_min(add_rn(excl, mex), pend)), static_cast<acc_t>(1));
         const auto counts = [&](const auto &str) {
             strata_counts(str, loc, Jr, excl, pend, nrm, eb, cnt, k0, N, dbg_cdf, st);
-            jbl = (lt == 0) ? 0 : str.count_le(c_beg);
+            if (!kF64 || warp * 32 * kItems < cnt) jbl = (lt == 0) ? 0 : str.count_le(c_beg);
             if (lane == 0 && tid != 0 && eb < cnt) jprev0 = str.count_le(c_prev);
             if (tid == 0) jprev0 = jbl;
         };

@@ -132,3 +132,15 @@ def test_gumbel_list_chunks(pf, n):
     for j in bad:
         g = oracle.gumbel_variates(29, 0, int(j), n)
         assert abs(g[want[j]] - g[anc[j]]) <= 1e-5 * max(1.0, abs(like[0]))
+
+
+@pytest.mark.parametrize("prec", ["ref64", "f32"])
+@pytest.mark.parametrize("x,y", [(10.5, 9.5), (10.499999, 9.500001), (-0.5, -1.5), (0.0, -0.25), (63.5, 31.75),
+                                 (1e-30, -1e-30), (70000.0, -5e5)])
+def test_pixels_at_half_integers(pf, prec, x, y):
+    """Particles without noise exactly on, and next to, the positions where a pixel ends."""
+    v = synth.make_video(64, 48, 2, 3, noise=8.0, seed=30)
+    f = pf.Filter(v.W, v.H, 37, 3, prec, init=(x, y), seed=31, sigma=(0.0, 0.0))
+    f.run(_cuda(v.frames))
+    _check_likelihoods(pf, f, prec, v.frames[-1], 3)
+    f.close()
