@@ -189,7 +189,7 @@ def _peaks():
         return 6800.0, "fallback"
 
 
-KERNEL_SOURCES = ("pf_step.cu", "pf_device.cuh", "pf_internal.h")
+KERNEL_SOURCES = ("pf_step.cu", "pf_device.cuh", "pf_ref64.cuh", "pf_internal.h")
 
 
 def _kernel_source_hash():
