@@ -16,6 +16,15 @@ __device__ __forceinline__ int ancestor_tracker(const AncestorLaunch &G, int b) 
     return lo;
 }
 
+// Rejection: offspring per CTA of a tracker of n particles (a multiple of 32).  Small trackers are
+// spread over the SMs (kRejectionSpread CTAs, four an SM, while a CTA keeps 32 offspring, four a
+// warp): F32 1000 particles in one CTA of at most kRejectionOffspring 77 us a frame, so 13.
+constexpr int kRejectionSpread = 608;
+__host__ __device__ inline int rejection_pool(int64_t n) {
+    const int64_t p = ((n + kRejectionSpread - 1) / kRejectionSpread + 31) / 32 * 32;
+    return p > kRejectionOffspring ? kRejectionOffspring : static_cast<int>(p);
+}
+
 __device__ __forceinline__ double log_uniform(uint32_t w, double) { return log(uniform_f64(w)); }
 __device__ __forceinline__ float log_uniform(uint32_t w, float) { return logf(uniform_f32(w)); }
 

@@ -14,12 +14,17 @@
 // candidate is kept (the loop is bounded whatever the weights).  The test runs in FP64 for
 // REF64 and FP32 for the others (L widened exactly from its stored type).
 //
-// Layout: CTA b takes kRejectionOffspring consecutive offspring as a pool its
-// kRejectionThreads threads share: each loop iteration is eight tries of every lane's
-// current offspring (their gathers in flight together), and a lane whose offspring is
-// decided takes the next undecided one from a shared counter.  A warp therefore stays busy until the pool is empty instead of waiting,
-// for each group of 32 offspring, for the largest of 32 geometric try counts; every
-// offspring's tries and decision are those of its own Philox stream either way.
+// Layout: CTA b takes rejection_pool(N) consecutive offspring as a pool its kRejectionThreads
+// threads share: each loop iteration is eight tries of every lane's current offspring (their
+// gathers in flight together), and a lane whose offspring is decided takes the next undecided
+// one from a shared counter, so a warp does not wait, for each group of 32 offspring, for the
+// largest of 32 geometric try counts.  Once the pool is empty the offspring still undecided
+// (one a thread at most) go to a list in shared memory, and each warp takes one at a time, 64
+// tries in order per iteration, two a lane: left to their own lanes, the last of a CTA's
+// offspring take as long as the whole pool before them.  Every offspring's tries and decision
+// are those of its own Philox stream either way.  Us a frame, 2048 a CTA without the list ->
+// rejection_pool(N) with it: F16 2^20 161 -> 129, 200003 91 -> 53, F32 30001 119 -> 28, BF16 5003
+// 119 -> 18, REF64 20003 100 -> 44.
 #include <math.h>
 
 #include "pf_ancestor.cuh"
@@ -35,6 +40,8 @@ __global__ void __launch_bounds__(kRejectionThreads) rejection_kernel(const Ance
     using acc_t = typename Prec<P>::acc_t;
     constexpr bool kF64 = sizeof(acc_t) == 8;
     __shared__ unsigned int s_next;   // next undecided offspring of the pool (local index)
+    __shared__ unsigned int s_left, s_take;          // listed offspring, and how many of them are taken
+    __shared__ int s_e[kRejectionThreads], s_i[kRejectionThreads];   // their pool indices and next tries
     const int b = static_cast<int>(blockIdx.x);
     const int g = ancestor_tracker(G, b);
     const int slot = __ldg(G.slots + g);
@@ -43,9 +50,10 @@ __global__ void __launch_bounds__(kRejectionThreads) rejection_kernel(const Ance
     const int64_t t = st->t;
     if (t <= 0 || (st->status & kStatusTimeout) || !G.frames[slot].active) return;
     const int N = static_cast<int>(T.N);
-    const int64_t j0 = static_cast<int64_t>(b - __ldg(G.cta_prefix + g)) * kRejectionOffspring;
-    const int pool = static_cast<int>(N - j0 < kRejectionOffspring ? N - j0 : kRejectionOffspring);
-    if (threadIdx.x == 0) s_next = kRejectionThreads;
+    const int per = rejection_pool(N);
+    const int64_t j0 = static_cast<int64_t>(b - __ldg(G.cta_prefix + g)) * per;
+    const int pool = static_cast<int>(N - j0 < per ? N - j0 : per);
+    if (threadIdx.x == 0) { s_next = kRejectionThreads; s_left = 0u; s_take = 0u; }
     __syncthreads();
     const lik_t *__restrict__ L = static_cast<const lik_t *>(T.pl[static_cast<int>((t + 1) & 1)]);
     const acc_t M = kF64 ? static_cast<acc_t>(st->M) : static_cast<acc_t>(st->M_f);
@@ -56,7 +64,7 @@ __global__ void __launch_bounds__(kRejectionThreads) rejection_kernel(const Ance
 
     int e = static_cast<int>(threadIdx.x);   // the lane's offspring (pool index); >= pool: none
     int i = 0;                               // its next try (a multiple of 8)
-    while (e < pool) {
+    while (e < pool && *const_cast<volatile unsigned int *>(&s_next) < static_cast<unsigned int>(pool)) {
         const int jj = static_cast<int>(j0) + e;
         const uint32_t tag = 6u + (static_cast<uint32_t>(jj) << 8);
         // eight tries at a time: proposals (four Philox blocks) and gathers first, all eight
@@ -90,6 +98,34 @@ __global__ void __launch_bounds__(kRejectionThreads) rejection_kernel(const Ance
             i = 0;
         } else {
             i += 8;
+        }
+    }
+    if (e < pool) {
+        const unsigned int at = atomicAdd(&s_left, 1u);
+        s_e[at] = e;
+        s_i[at] = i;
+    }
+    __syncthreads();
+    const unsigned int left = s_left;
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        unsigned int at = 0u;
+        if (lane == 0) at = atomicAdd(&s_take, 1u);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (at >= left) break;
+        const int jj = static_cast<int>(j0) + s_e[at];
+        const uint32_t tag = 6u + (static_cast<uint32_t>(jj) << 8);
+        for (int i0 = s_i[at];; i0 += 64) {          // (a multiple of 8; ends at R at the latest)
+            const int x = i0 + 2 * lane;             // the lane's tries x and x + 1
+            const uint4 w = philox4x32_10(make_uint4(static_cast<uint32_t>(x >> 1), tctr, tag, trk_id), key_lo, key_hi);
+            const int ka = x == 0 ? jj : static_cast<int>(__umulhi(w.x, n)), kb = static_cast<int>(__umulhi(w.z, n));
+            const acc_t la = x < R ? to_acc(L[ka]) : acc_t{}, lb = x + 1 < R ? to_acc(L[kb]) : acc_t{};
+            const bool da = x < R && (log_uniform_le<acc_t>(w.y, la - M) || x + 1 >= R);
+            const bool db = x + 1 < R && (log_uniform_le<acc_t>(w.w, lb - M) || x + 2 >= R);
+            const uint32_t mask = __ballot_sync(0xffffffffu, da || db);
+            if (mask == 0u) continue;
+            if (lane == __ffs(static_cast<int>(mask)) - 1) T.anc[jj] = da ? ka : kb;
+            break;
         }
     }
 }

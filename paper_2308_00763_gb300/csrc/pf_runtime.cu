@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "pf.h"
+#include "pf_ancestor.cuh"
 #include "pf_internal.h"
 #include "pf_host.h"
 
@@ -259,7 +260,7 @@ static pf_status engine_init(Engine &e, const pf_config *cfgs, int n, void *stre
         }
         if (given) {
             const int s = c.resampler == PF_RESAMPLE_GUMBEL ? 0 : c.resampler == PF_RESAMPLE_METROPOLIS ? 1 : 2;
-            const int per = s == 0 ? kGumbelOffspring : s == 1 ? kMetropolisThreads : kRejectionOffspring;
+            const int per = s == 0 ? kGumbelOffspring : s == 1 ? kMetropolisThreads : rejection_pool(static_cast<int64_t>(N));
             const int64_t ctas = aprefix[s].back() + (N + per - 1) / per;
             if (ctas > 0x7fffffff) return PF_ERR_ARG;
             atab[s].push_back(i);

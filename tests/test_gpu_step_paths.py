@@ -144,3 +144,25 @@ def test_pixels_at_half_integers(pf, prec, x, y):
     f.run(_cuda(v.frames))
     _check_likelihoods(pf, f, prec, v.frames[-1], 3)
     f.close()
+
+
+@pytest.mark.parametrize("n,tries", [(31, 0), (33, 0), (19456, 0), (19457, 0), (155649, 0), (5000, 63), (5000, 64),
+                                     (5000, 65), (5000, 129), (200003, 9)])
+def test_rejection_pools_and_lists(pf, n, tries):
+    """Pools of less than a thread's share, at the sizes where a pool grows, and beyond the threads
+    of a CTA; try limits around the 64 tries that a warp takes at once."""
+    v = synth.make_video(128, 128, 3, 5, noise=5.0, seed=32)
+    f = pf.Filter(v.W, v.H, n, 5, "f32", init=tuple(v.centres[0]), seed=33, flags=pf.PF_FLAG_DEBUG_ARRAYS,
+                  resampler="rejection", resampler_steps=tries)
+    fr = _cuda(v.frames)
+    f.run(fr[:2])
+    st = f.get_state()
+    f.step(fr[2])
+    anc = f.debug(0).astype(np.int64)
+    f.close()
+    L, M, t = st["L"].astype(np.float64), float(st["max_l"]), int(st["t"]) - 1
+    tries = tries or 4096
+    bad = np.nonzero(anc != oracle.resample_rejection(L, M, 33, t, 0, "f32", tries))[0]
+    assert bad.size <= max(1, n // 1000)   # (tests within rounding of their threshold)
+    for j in bad:
+        assert min(oracle.rejection_trace(L, M, 33, t, int(j), 0, tries)[1]) <= 1e-4
