@@ -1,6 +1,7 @@
 """Build the sm_103a library ``_build/libpf_gb300.so`` from ``csrc/*.cu`` with nvcc.
 
-Each translation unit is compiled in parallel, then linked with -shared.  The build is
+The FP64 function tables are written first (:mod:`.ref64_tables`), then each translation unit
+is compiled in parallel and linked with -shared.  The build is
 skipped when the library is newer than every source and header.
 """
 from __future__ import annotations
@@ -10,6 +11,11 @@ import os
 import shutil
 import subprocess
 import sys
+
+try:
+    from . import ref64_tables
+except ImportError:        # run as a program
+    import ref64_tables
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -32,7 +38,7 @@ def sources():
 
 def deps():
     return sources() + sorted(glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))) + [
-        os.path.join(ROOT, "include", "pf.h"), os.path.abspath(__file__)]
+        os.path.join(ROOT, "include", "pf.h"), os.path.abspath(__file__), os.path.abspath(ref64_tables.__file__)]
 
 
 STUDY_THREADS = (128, 256, 512, 1024)   # threads per CTA of the step kernel's study builds
@@ -78,8 +84,9 @@ def build(force: bool = False, verbose: bool = False, extra=(), threads: int | N
     bdir = os.path.dirname(lib)
     os.makedirs(bdir, exist_ok=True)
     cc = nvcc()
+    ref64_tables.write(os.path.join(bdir, "ref64_tables.inc"))
     flags = [ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"),
-             "--expt-relaxed-constexpr", *extra]
+             "-I", bdir, "--expt-relaxed-constexpr", *extra]
     if checked:
         flags.append("-DPF_CHECKED")
     elif naive:

@@ -186,9 +186,6 @@ struct StepLaunch {
 };
 
 // Host entry points into the kernel translation unit.
-// Upload what the kernels of a precision read besides their arguments (the FP64 tables) to the
-// current device, once per device; waits for `stream`.  Before the first launch.
-int step_prepare(int precision, void *stream);
 int launch_step(int precision, const StepLaunch &L, int grid, void *stream);
 // The pull family's kernels after launch_step on the same stream: the multinomial
 // trackers' CDF kernel (when with_cdf), then the pull kernel (the offspring of the

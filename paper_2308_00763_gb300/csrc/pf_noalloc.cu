@@ -172,7 +172,6 @@ extern "C" pf_status pf_step_frame_noalloc(const pf_config *cfg, const pf_state_
     unsigned char *scr = nullptr;
     pf_status s = scratch_for_current_device(&dev, &scr);
     if (s != PF_OK) return s;
-    if (step_prepare(c.precision, cuda_stream) != 0) return PF_ERR_CUDA;
     constexpr ScratchLayout LY = layout();
 
     // descriptor of the tracker: the caller's buffers are the ping-pong slots of frame t

@@ -8,8 +8,9 @@
 // ACM TOMS 16, 1990; angle addition for sine and cosine) need 19 FP64 operations a Box-Muller
 // pair and 9 an exponential; field extraction, scaling by powers of two and the conversions to
 // and from FP32 (which run at the FP64 rate) are integer operations on the words.
-// The tables (113 KB) hold correctly rounded values, computed in extended precision on the host
-// when a device first needs them.  The argument of the logarithm and the angle have 24 bits
+// The tables (113 KB) hold correctly rounded values, written by the build (ref64_tables.py) and
+// compiled in as initialised data: every context that loads the library has them, with no upload
+// to order against a launch and no record of who has made one.  The argument of the logarithm and the angle have 24 bits
 // (the generator's uniforms), which the splits below use.  Errors, against extended precision
 // over all 2^23 uniforms: radius below 0.86 ulp (as with the library's log and sqrt), sine and
 // cosine below 1.7e-16; exponential below 0.51 ulp on [-700, 0].  Measured us a frame, library functions ->
@@ -30,7 +31,9 @@ struct Ref64Tables {
 };
 constexpr int kLnUpper = 424;   // first interval whose centre is above sqrt 2
 
-__device__ Ref64Tables g_ref64;
+__device__ const Ref64Tables g_ref64 = {
+#include "ref64_tables.inc"
+};
 
 // Exact conversions of normal values by their words.
 __device__ __forceinline__ double widen_bits(float f) {

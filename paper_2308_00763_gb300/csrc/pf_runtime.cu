@@ -358,7 +358,6 @@ static pf_status engine_init(Engine &e, const pf_config *cfgs, int n, void *stre
         if (tabs[s]->n > 0)
             err = cudaMemcpyAsync(tabs[s]->d, atab[s].data(), sizeof(int32_t) * atab[s].size(), cudaMemcpyHostToDevice,
                                   e.stream);
-    if (err == cudaSuccess && step_prepare(e.prec, e.stream) != 0) err = cudaErrorUnknown;
     if (err == cudaSuccess) err = cudaMemsetAsync(e.d_ticket, 0, sizeof(uint32_t), e.stream);
     e.h_gather = reinterpret_cast<double *>(e.h_states + n);
     e.d_init = reinterpret_cast<TrackerState *>(e.d_arena + init_off);

@@ -202,7 +202,6 @@ pf_status engine_init(pf_server *S, int prec) {
     if (e.prec >= 0) return PF_OK;
     const int cap = S->cfg.max_streams;
     cudaError_t err = cudaStreamCreateWithFlags(&e.stream, cudaStreamNonBlocking);
-    if (err == cudaSuccess && step_prepare(prec, e.stream) != 0) err = cudaErrorUnknown;
     if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&e.d_trk), sizeof(TrackerDev) * cap);
     if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&e.d_states), sizeof(TrackerState) * cap);
     if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&e.d_ticket), sizeof(uint32_t));

@@ -154,7 +154,6 @@ extern "C" pf_status pf_shard_create(const pf_config *cfg, int32_t rank, int32_t
     const size_t o_cdf = take(pb * count + 16), o_anc = take(sizeof(int32_t) * count + 16);
     cudaError_t err = cudaMalloc(reinterpret_cast<void **>(&h->d_arena), off);
     if (err == cudaSuccess) err = cudaMemsetAsync(h->d_arena, 0, off, h->stream);
-    if (err == cudaSuccess && step_prepare(h->prec, h->stream) != 0) err = cudaErrorUnknown;
     if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&h->d_trk), sizeof(TrackerDev));
     if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&h->d_frame), sizeof(FrameRef));
     if (err == cudaSuccess) err = cudaMalloc(reinterpret_cast<void **>(&h->d_ticket), sizeof(uint32_t));

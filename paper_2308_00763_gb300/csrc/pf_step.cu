@@ -2319,50 +2319,6 @@ int slots_of(int precision) {
 }
 }  // namespace
 
-// The FP64 tables, each entry rounded once from extended precision.
-static Ref64Tables::Ln split_ln(float c, long double v) {
-    const long double hi = rintl(v * 4398046511104.0L) / 4398046511104.0L;   // a multiple of 2^-42
-    return Ref64Tables::Ln{c, static_cast<float>(v - hi), static_cast<double>(hi)};
-}
-static bool fill_ref64_tables(Ref64Tables &t) {
-    const long double pi = 3.14159265358979323846264338327950288L, ln2 = 0.693147180559945309417232121458176568L;
-    for (int i = 0; i < 2048; ++i) {
-        t.turn_hi[i] = double2{static_cast<double>(cosl(pi * i / 4096)), static_cast<double>(sinl(pi * i / 4096))};
-        t.turn_lo[i] = double2{static_cast<double>(cosl(pi * i / 8388608)), static_cast<double>(sinl(pi * i / 8388608))};
-        const long double e = exp2l(static_cast<long double>(i) / 2048);
-        t.ex[i].x = static_cast<double>(e);
-        t.ex[i].y = static_cast<double>(e - t.ex[i].x);
-    }
-    for (int i = 0; i < 32; ++i) t.eln2[i] = split_ln(0.0f, -ln2 * i);
-    for (int j = 0; j < 1024; ++j) {
-        // the last interval takes c = 1/2, so that ln u keeps its relative accuracy next to u = 1
-        const float c = j == 1023 ? 0.5f : static_cast<float>(1.0 / (1.0 + (j + 0.5) / 1024));
-        const long double cl = c;
-        t.ln[j] = split_ln(c, -logl(j >= kLnUpper ? 2 * cl : cl));
-    }
-    return true;
-}
-static const Ref64Tables &ref64_tables() {
-    static Ref64Tables t;
-    static const bool filled = fill_ref64_tables(t);
-    (void)filled;
-    return t;
-}
-
-int step_prepare(int precision, void *stream) {
-    if (precision != 0) return 0;
-    static std::atomic<int> ready[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return -1; }
-    if (dev >= 0 && dev < 64 && ready[dev].load(std::memory_order_acquire)) return 0;
-    const cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t err = cudaMemcpyToSymbolAsync(g_ref64, &ref64_tables(), sizeof(Ref64Tables), 0, cudaMemcpyHostToDevice, s);
-    if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-    if (err != cudaSuccess) { cudaGetLastError(); return -1; }
-    if (dev >= 0 && dev < 64) ready[dev].store(1, std::memory_order_release);
-    return 0;
-}
-
 int step_tile_size(int precision, int64_t n) {
     const int64_t slots = slots_of(precision);
     // a tracker that cannot fill half the device with full tiles keeps full tiles (in a

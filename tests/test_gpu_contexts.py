@@ -1,0 +1,82 @@
+"""A second CUDA context on the device: it has its own copy of everything the library keeps in
+device variables.  The same calls there give the bits of the first context's.  (In a child
+process, which makes the context with the driver's own calls and takes it down again.)"""
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+_CHILD = r"""
+import ctypes, sys
+import numpy as np
+import paper_2308_00763_gb300 as pf
+from paper_2308_00763_gb300 import synth
+
+cu = ctypes.CDLL("libcuda.so.1")
+
+
+def check(rc, what):
+    if rc != 0:
+        raise RuntimeError("%s: %d" % (what, rc))
+
+
+check(cu.cuInit(0), "cuInit")
+pf.lib(build_if_missing=True)
+v = synth.make_video(96, 80, 3, 4, noise=5.0, seed=51)
+
+
+def engine(prec):
+    f = pf.Filter(v.W, v.H, 3001, 4, prec, stream=0, init=tuple(v.centres[0]), seed=52)
+    for frame in v.frames:
+        f.step(frame)
+    st = f.get_state()
+    est = f.estimates(0, v.T)
+    f.close()
+    return [st["x"], st["y"], st["L"], np.asarray(est)]
+
+
+def in_second_context(call):
+    ctx = ctypes.c_void_p()
+    dev = ctypes.c_int()
+    check(cu.cuDeviceGet(ctypes.byref(dev), 0), "cuDeviceGet")
+    check(cu.cuCtxCreate_v2(ctypes.byref(ctx), 0, dev), "cuCtxCreate")   # (made current)
+    try:
+        return call()
+    finally:
+        check(cu.cuCtxDestroy_v2(ctx), "cuCtxDestroy")
+
+
+def same(a, b):
+    for p, q in zip(a, b):
+        assert np.array_equal(np.asarray(p).view(np.uint8), np.asarray(q).view(np.uint8))
+
+
+def run_engine(prec):
+    first = engine(prec)
+    same(first, in_second_context(lambda: engine(prec)))
+    same(first, engine(prec))     # (and the first context is as it was)
+
+
+globals()["run_" + sys.argv[1]](sys.argv[2])
+print("same bits")
+"""
+
+
+def _child(kind, prec):
+    env = dict(os.environ, PYTHONPATH=ROOT + os.pathsep + os.environ.get("PYTHONPATH", ""))
+    p = subprocess.run([sys.executable, "-c", _CHILD, kind, prec], cwd=ROOT, env=env, capture_output=True, text=True,
+                       timeout=300)
+    assert p.returncode == 0 and "same bits" in p.stdout, p.stdout + p.stderr
+
+
+@pytest.mark.parametrize("prec", ["ref64", "f32"])
+def test_filter_in_a_second_context(prec):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    _child("engine", prec)
