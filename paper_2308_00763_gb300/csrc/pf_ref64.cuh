@@ -5,24 +5,28 @@
 // its FP64 operations, two thirds of which were the math library's log, sqrt, sincospi and exp.
 // Table-driven forms (P. T. P. Tang, "Table-driven implementation of the exponential function
 // in IEEE floating-point arithmetic", ACM TOMS 15, 1989, and "... of the logarithm function",
-// ACM TOMS 16, 1990; angle addition for sine and cosine) need 19 FP64 operations a Box-Muller
+// ACM TOMS 16, 1990; angle addition for sine and cosine) need 21 FP64 operations a Box-Muller
 // pair and 9 an exponential; field extraction, scaling by powers of two and the conversions to
 // and from FP32 (which run at the FP64 rate) are integer operations on the words.
-// The tables (113 KB) hold correctly rounded values, written by the build (ref64_tables.py) and
+// The tables (104 KB) hold correctly rounded values, written by the build (ref64_tables.py) and
 // compiled in as initialised data: every context that loads the library has them, with no upload
-// to order against a launch and no record of who has made one.  The argument of the logarithm and the angle have 24 bits
-// (the generator's uniforms), which the splits below use.  Errors, against extended precision
-// over all 2^23 uniforms: radius below 0.86 ulp (as with the library's log and sqrt), sine and
-// cosine below 1.7e-16; exponential below 0.51 ulp on [-700, 0].  Measured us a frame, library functions ->
-// tables: 2^20 particles 375 -> 227, 200003 231 -> 134.
+// to order against a launch and no record of who has made one.  The argument of the logarithm and
+// the angle have 24 bits (the generator's uniforms), which the splits below use.
+// Largest errors in ulp of the value (and their root mean square), over all 2^23 uniforms, and
+// over 2^22 arguments of the exponential in [-30, 0], CUDA's functions -> these:
+//   radius        0.852 (0.3254) -> 0.852 (0.3254)
+//   sine, cosine  1.476 (0.3610) -> 1.093 (0.2888)
+//   exponential   0.888 (0.3017) -> 0.501 (0.2887)
+// Measured us a frame, library functions -> tables: 2^20 particles 375 -> 227, 200003 231 -> 134.
 #pragma once
 #include <stdint.h>
 
 namespace pfk {
 
 struct Ref64Tables {
-    double2 turn_hi[2048];   // (cos, sin)(2 pi i / 2^13): the quadrant's top 11 bits
-    double2 turn_lo[2048];   // (cos, sin)(2 pi i / 2^24): its low 11 bits
+    double2 turn_hi[1024];   // (cos, sin)(2 pi i / 2^13): an octant's top 10 bits
+    float2 turn_rest[1024];  // ... their rounding errors
+    double2 turn_lo[2048];   // (cos - 1, sin)(2 pi i / 2^24): its low 11 bits
     double2 ex[2048];        // 2^(i / 2048) and its rounding error
     // per mantissa interval of [1, 2): c ~ 1 / centre with 24 bits, and -ln c (from interval
     // kLnUpper on -ln 2c: the mantissa is halved) as a multiple of 2^-42 and the rest
@@ -74,13 +78,19 @@ __device__ __forceinline__ void box_muller_table(uint32_t wa, uint32_t wb, doubl
     double s = y * g;
     s = fma(fma(-s, s, y), h, s);
     s = fma(fma(-s, s, y), h, s);
-    // u_b = v / 2^24: quadrant, then the angle's two halves
+    // u_b = v / 2^24, v odd: quadrant, the angle's distance to the nearer axis (below an octant, so
+    // that neither value is a difference of larger ones), and that angle's two halves
     const uint32_t v = (wb >> 8) | 1u, rem = v & 0x3fffffu, quad = v >> 22;
-    const double2 a = __ldg(&g_ref64.turn_hi[rem >> 11]), b = __ldg(&g_ref64.turn_lo[rem & 2047u]);
-    const double co = s * fma(a.x, b.x, -(a.y * b.y)), si = s * fma(a.y, b.x, a.x * b.y);
-    const bool odd = (quad & 1u) != 0u;
-    nx = flip_bits(odd ? si : co, (quad == 1u || quad == 2u) ? 0x80000000u : 0u);
-    ny = flip_bits(odd ? co : si, quad >= 2u ? 0x80000000u : 0u);
+    const bool far = rem > 0x200000u;
+    const uint32_t o = far ? 0x400000u - rem : rem;
+    const double2 a = __ldg(&g_ref64.turn_hi[o >> 11]), b = __ldg(&g_ref64.turn_lo[o & 2047u]);
+    const float2 t = __ldg(&g_ref64.turn_rest[o >> 11]);
+    // cos(a + b) = cos a + (rest + cos a (cos b - 1) - sin a sin b), the sine likewise
+    const double ca = s * (a.x + fma(a.x, b.x, fma(-a.y, b.y, widen_bits(t.x))));
+    const double sa = s * (a.y + fma(a.y, b.x, fma(a.x, b.y, widen_bits(t.y))));
+    const bool swap = far != ((quad & 1u) != 0u);
+    nx = flip_bits(swap ? sa : ca, (quad == 1u || quad == 2u) ? 0x80000000u : 0u);
+    ny = flip_bits(swap ? ca : sa, quad >= 2u ? 0x80000000u : 0u);
 }
 
 // exp(d) for |d| < 700 (the caller's test is on the high word): 2^(k + i/2048) (1 + p(r)).

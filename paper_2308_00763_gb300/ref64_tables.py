@@ -15,7 +15,7 @@ LN_UPPER = 424   # first logarithm interval whose centre is above sqrt 2 (kLnUpp
 
 
 def _sin_cos(a: Decimal):
-    """Sine and cosine of 0 <= a < 2 by their power series."""
+    """Sine and cosine of 0 <= a < 1 by their power series."""
     s, c, term, k = Decimal(0), Decimal(0), Decimal(1), 0
     while abs(term) > Decimal("1e-58"):
         sign = -1 if k & 2 else 1
@@ -51,9 +51,17 @@ def _ln(c: float, v: Decimal) -> str:
 def rows():
     """The members of Ref64Tables in order, each a list of entries."""
     getcontext().prec = 60
-    def turns(n, steps):
-        return [_pair(float(c), float(s)) for s, c in (_sin_cos(2 * PI * i / steps) for i in range(n))]
-    hi, lo = turns(2048, 1 << 13), turns(2048, 1 << 24)
+    hi, hi_rest = [], []
+    for i in range(1024):
+        s, c = _sin_cos(PI * i / 4096)
+        (c0, c1), (s0, s1) = _with_rest(c), _with_rest(s)
+        hi.append(_pair(c0, s0))
+        hi_rest.append("{%sf, %sf}" % (_f32(c1).hex(), _f32(s1).hex()))
+    lo = []
+    for i in range(2048):
+        s, _ = _sin_cos(PI * i / 8388608)
+        h, _ = _sin_cos(PI * i / 16777216)
+        lo.append(_pair(float(-2 * h * h), float(s)))
     ln2 = Decimal(2).ln()
     ex = []
     for i in range(2048):
@@ -65,7 +73,7 @@ def rows():
         c = 0.5 if j == 1023 else _f32(1.0 / (1.0 + (j + 0.5) / 1024))
         ln.append(_ln(c, -(Decimal(c) * (2 if j >= LN_UPPER else 1)).ln()))
     eln2 = [_ln(0.0, -ln2 * i) for i in range(32)]
-    return [hi, lo, ex, ln, eln2]
+    return [hi, hi_rest, lo, ex, ln, eln2]
 
 
 def write(path: str) -> str:

@@ -166,3 +166,32 @@ def test_rejection_pools_and_lists(pf, n, tries):
     assert bad.size <= max(1, n // 1000)   # (tests within rounding of their threshold)
     for j in bad:
         assert min(oracle.rejection_trace(L, M, 33, t, int(j), 0, tries)[1]) <= 1e-4
+
+
+def test_fp64_draws_are_accurate_next_to_the_axes(pf):
+    """Every draw of a frame around the origin relative to its own size, against extended
+    precision from the generator's words.  In units of 2^-52: the radius is within 0.852, the sine
+    or cosine within 1.093, and their product's rounding adds 0.5, so 2.45; second-order terms
+    and the reference (64 bits or more) stay below 0.05.  (Drift 0 and sigma 1 are exact.)"""
+    ld = np.longdouble
+    v = synth.make_video(64, 64, 1, 3, noise=5.0, seed=41)
+    n = 1 << 20
+    f = pf.Filter(64, 64, n, 3, "ref64", init=(0.0, 0.0), seed=42)
+    f.run(_cuda(v.frames))
+    st = f.get_state()
+    f.close()
+    ctr = np.zeros((n // 2, 4), np.uint32)
+    ctr[:, 0] = np.arange(n // 2)
+    w = oracle.philox(ctr, 42).reshape(n, 2)
+    m = 2 * (w >> 9).astype(np.int64) + 1                    # u = m / 2^24
+    rad = np.sqrt(-2 * np.log(m[:, 0].astype(ld) / (1 << 24)))
+    quad, rem = m[:, 1] >> 22, m[:, 1] & 0x3fffff
+    far = rem > 1 << 21                                      # nearer to the quarter's end
+    pi = ld("3.14159265358979323846264338327950288")
+    a = pi * np.where(far, (1 << 22) - rem, rem).astype(ld) / (1 << 23)
+    swap = far != (quad % 2 == 1)
+    c, s = np.where(swap, np.sin(a), np.cos(a)), np.where(swap, np.cos(a), np.sin(a))
+    want_x = np.where((quad == 1) | (quad == 2), -c, c) * rad
+    want_y = np.where(quad >= 2, -s, s) * rad
+    for got, want in ((st["x"], want_x), (st["y"], want_y)):
+        assert np.abs((got - want) / want).max() <= 2.5 * 2.0 ** -52
