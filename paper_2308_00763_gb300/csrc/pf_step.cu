@@ -657,19 +657,50 @@ __device__ __forceinline__ uint32_t warp_disk_sum(const FrameView &f, const int8
     return __reduce_add_sync(0xffffffffu, s);
 }
 
+// The likelihood of a pixel straight from the frame, by one lane.
+template <int P, typename L>
+__device__ __forceinline__ L direct_likelihood(const TrackerDev &T, const FrameView &f, const int8_t *w, int px, int py) {
+    using acc_t = typename Prec<P>::acc_t;
+    if constexpr (Prec<P>::kHalf) {
+        return half_lik<L>(T).at(f, w, px, py);
+    } else {
+        constexpr bool kF64 = sizeof(acc_t) == 8;
+        return lik_from_sum<acc_t>(disk_sum(f, w, px, py), kF64 ? static_cast<acc_t>(T.c1) : static_cast<acc_t>(T.c1f),
+                                   kF64 ? static_cast<acc_t>(T.c2 * T.D) : static_cast<acc_t>(T.c2Df),
+                                   kF64 ? static_cast<acc_t>(T.den) : static_cast<acc_t>(T.denf));
+    }
+}
+
 // The direct route of the offspring loop: the likelihoods of pixels outside the tile's window,
-// straight from the frame, by all the lanes of `act` that are in the loop's iteration together
-// (miss: which of the lane's two particles need one, 1 and 2).  The lanes take the template's
-// rows of one particle after another, so a particle costs one or two round trips of loads
-// in flight together; its own lane alone read |D| pixels in a nearly serial chain, microseconds
+// straight from the frame, for all the lanes of `act` that are in the loop's iteration together
+// (miss: which of the lane's two particles need one, 1 and 2).
+// Few of them (a draw beyond the window's 3.5 sigma): the lanes take the template's rows of one
+// particle after another, so a particle costs one or two round trips of loads in flight
+// together; its own lane alone read |D| pixels in a nearly serial chain, microseconds
 // that the whole block waited for at the next barrier.  The sums are HalfLik::at's (rows left
 // to right, row sums top to bottom) and disk_sum's, so the bits are.  F16, the paper's motion
 // model at 65536 particles (about four such particles a tile): 20.1 -> 18.6 us a frame.
+// Many (no window fits a table: every draw, from about 10 px of noise on): each lane its own, where
+// none waits for another's and the chains of a warp run side by side.  Every particle of 65536,
+// noise 10, radius 5, one after another -> each lane its own: F16 807 -> 108 us a frame, F32 367 ->
+// 98, REF64 409 -> 99; 200003, radius 40: F16 15 930 -> 5390, F32 10 970 -> 4570.
+// So a warp's 64 particles one after another cost 7.5 (F16) and 3.7 (F32) times as much as at once
+// with 81 pixels, 3.0 and 2.4 with 5025: the line lies at an eighth of them in half and
+// at a quarter otherwise.
+template <int P> constexpr int kDirectShare = Prec<P>::kHalf ? 4 : 2;   // per lane in the iteration
 template <int P, typename L>
 __device__ __forceinline__ void direct_likelihoods(const TrackerDev &T, const FrameView &f, const int8_t *w, unsigned act,
                                                    int miss, int px0, int py0, int px1, int py1, L &l0, L &l1) {
     using acc_t = typename Prec<P>::acc_t;
     const int lane = threadIdx.x & 31, n = __popc(act), rank = __popc(act & ((1u << lane) - 1u));
+    if (kDirectShare<P> * (__popc(__ballot_sync(act, miss != 0)) + __popc(__ballot_sync(act, miss == 3))) > n) {
+        for (int side = 1; side <= 2; ++side) {
+            if (!(miss & side)) continue;
+            const L v = direct_likelihood<P, L>(T, f, w, side == 1 ? px0 : px1, side == 1 ? py0 : py1);
+            if (side == 1) l0 = v; else l1 = v;
+        }
+        return;
+    }
     const int nrow = 2 * f.r + 1;
     for (unsigned left; (left = __ballot_sync(act, miss != 0)) != 0u;) {
         const int src = __ffs(static_cast<int>(left)) - 1;

@@ -195,3 +195,17 @@ def test_fp64_draws_are_accurate_next_to_the_axes(pf):
     want_y = np.where(quad >= 2, -s, s) * rad
     for got, want in ((st["x"], want_x), (st["y"], want_y)):
         assert np.abs((got - want) / want).max() <= 2.5 * 2.0 ** -52
+
+
+@pytest.mark.parametrize("prec,accum32", [("ref64", 0), ("f32", 0), ("f16", 0), ("f16", 1), ("bf16", 0)])
+@pytest.mark.parametrize("n,r,sigma", [(40001, 0, (5.0, 2.0)), (40001, 12, (5.0, 2.0)), (70, 5, (5.0, 2.0)),
+                                       (5001, 3, (40.0, 30.0)), (7, 5, (40.0, 40.0))])
+def test_direct_route_of_few_and_of_all(pf, prec, accum32, n, r, sigma):
+    """Production trackers (no debug arrays): a few draws beyond a window of 3.5 sigma, which the lanes
+    of a warp score together, and noise that no window fits, where each lane scores its own."""
+    v = synth.make_video(200, 150, 3, 6, noise=8.0, seed=43)
+    flags = pf.PF_FLAG_ACCUM32 if accum32 else 0
+    f = pf.Filter(v.W, v.H, n, r, prec, init=tuple(v.centres[0]), seed=44, sigma=sigma, flags=flags)
+    f.run(_cuda(v.frames))
+    _check_likelihoods(pf, f, prec, v.frames[-1], r, flags)
+    f.close()
