@@ -770,7 +770,6 @@ struct __align__(16) StepSmem {
         // of two neighbouring cells
         __half2 term2[P == 2 ? kRoiMax / 2 : 1];
     } u;
-    alignas(16) uint16_t map[kMapMax];   // ancestor (tile element + 1) of each offspring
     alignas(16) int warp_imax[kWarps];
     alignas(16) acc_t warp_sum[kWarps];
     alignas(16) acc_t warp_max[kWarps];
@@ -792,8 +791,8 @@ struct __align__(16) StepSmem {
     TrackerDev trk;
     TrackerState st;
     FrameRef fr;
-    // last: only the step mode allocates them (see counts_array and row_words)
-    alignas(16) uint32_t rows[Tr::kHalf ? kRowWords : 4];   // half form: row sums of the table's rows
+    alignas(16) uint16_t map[kMapMax];   // ancestor (tile element + 1) of each offspring
+    // last: only the step mode allocates it (see counts_array and row_words)
     alignas(16) int32_t J[kTile];
 };
 
@@ -1159,14 +1158,20 @@ template <int P, int kMode>
 __device__ __forceinline__ int32_t *counts_array(StepSmem<P> &sm) {
     return kMode == kModeStep ? sm.J : reinterpret_cast<int32_t *>(sm.map);
 }
-// The words of the table's row sums: their own array in the step mode, in the pull mode the map,
-// which has no use there but for the ancestors' indices when debug arrays are on (24 KB less shared memory, which the L1 keeps for its searches and gathers).
+// Where the table's row sums lie while it is built.  In the step mode in J's memory, not written
+// before the table is read, and, if there are more, from the map's second half on, which is
+// cleared again behind them.  (An array of their own, 24 KB more a CTA, left the L1 28 KB an SM of
+// 92: F16, noise 40, 65536 particles, radius 5, all scored from the frame, 297 us a frame against
+// 202; 2^20 722 against 456; the same at noise 1.)  In the pull mode the map, which has no use there
+// but for the ancestors' indices when debug arrays are on.
 template <int P, int kMode>
-__device__ __forceinline__ uint32_t *row_words(StepSmem<P> &sm) {
-    return kMode == kModeStep ? sm.rows : reinterpret_cast<uint32_t *>(sm.map);
+__device__ __forceinline__ uint32_t *row_words(StepSmem<P> &sm, int words) {
+    static_assert(offsetof(StepSmem<P>, J) == offsetof(StepSmem<P>, map) + sizeof(sm.map), "the map's end and J are one piece");
+    uint32_t *const m = reinterpret_cast<uint32_t *>(sm.map);
+    return kMode != kModeStep ? m : m + kMapMax / 2 - (words > kTile ? kRowWords - kTile : 0);
 }
 template <int P, int kMode> constexpr size_t smem_bytes() {
-    return kMode == kModeStep ? sizeof(StepSmem<P>) : offsetof(StepSmem<P>, rows);
+    return kMode == kModeStep ? sizeof(StepSmem<P>) : offsetof(StepSmem<P>, J);
 }
 static_assert(sizeof(uint16_t) * kMapMax == sizeof(int32_t) * kTile, "J fits the map's memory");
 
@@ -1186,14 +1191,14 @@ static_assert(sizeof(uint16_t) * kMapMax == sizeof(int32_t) * kTile, "J fits the
 // particles r = 12 18.8 -> 16.1; F16 2^20 particles r = 5 21.8 -> 22.0 (there the tiles build
 // their tables while they wait for their predecessors).
 template <int P, int kMode, bool kPair>
-__device__ __forceinline__ void table_by_rows(StepSmem<P> &sm, int rw, int pw, int ww, int wh, int band,
+__device__ __forceinline__ void table_by_rows(StepSmem<P> &sm, int rw, int pw, int ww, int wh, int band, int words,
                                               TrackerState *st) {
     (void)st;
     using H = typename Prec<P>::pos_t;
     using R = typename std::conditional<kPair, __half2, float>::type;
     const TrackerDev &T = sm.trk;
     const int r = T.r, ncls = T.ncls, tid = threadIdx.x;
-    R *rows = reinterpret_cast<R *>(row_words<P, kMode>(sm));
+    R *rows = reinterpret_cast<R *>(row_words<P, kMode>(sm, words));
     const auto zero = [] { if constexpr (kPair) return __float2half2_rn(0.0f); else return 0.0f; };
     const auto add = [](R a, R b) { if constexpr (kPair) return __hadd2(a, b); else return a + b; };
     const auto term = [&](int i) {
@@ -1255,7 +1260,7 @@ __device__ __forceinline__ void cdf_search(const TrackerDev &T, const typename P
                                            StepSmem<P> &sm, TrackerState *st) {
     using A = typename Prec<P>::acc_t;
     (void)st;
-    constexpr int kCoarse = static_cast<int>(offsetof(StepSmem<P>, map) / sizeof(A));
+    constexpr int kCoarse = static_cast<int>(offsetof(StepSmem<P>, warp_imax) / sizeof(A));
     constexpr int kVec = 16 / static_cast<int>(sizeof(A));   // elements a 16-byte load
     const int N = static_cast<int>(T.N), n8 = static_cast<int>((T.N + 7) >> 3), n64 = static_cast<int>((T.N + 63) >> 6);
     const A *c64 = static_cast<const A *>(T.cdf64), *c8 = static_cast<const A *>(T.cdf8), *c1 = static_cast<const A *>(T.cdf);
@@ -1756,10 +1761,18 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             by_rows = (paired || !hk.half_acc) && (band == wh || band >= 4) && by_row < by_cell &&
                       (kMode == kModeStep || (kMode == kModePull && !T.dbg_anc));
             if (by_rows) {
+                const int words = T.ncls * pw * (band + 2 * r);
                 if constexpr (P == 2) {
-                    if (paired) table_by_rows<P, kMode, true>(sm, rw, pw, ww, wh, band, st);
+                    if (paired) table_by_rows<P, kMode, true>(sm, rw, pw, ww, wh, band, words, st);
                 }
-                if (!paired) table_by_rows<P, kMode, false>(sm, rw, pw, ww, wh, band, st);
+                if (!paired) table_by_rows<P, kMode, false>(sm, rw, pw, ww, wh, band, words, st);
+                if constexpr (kMode == kModeStep) {
+                    if (words > kTile) {   // the map's second half was in use
+                        __syncthreads();
+                        reinterpret_cast<uint4 *>(sm.map)[kThreads + tid] = make_uint4(0u, 0u, 0u, 0u);
+                    }
+                    if (lt == 0) __syncthreads();   // (before J and the map are written; else the lookback's)
+                }
             }
         }
         if (paired && !by_rows) {

@@ -209,3 +209,29 @@ def test_direct_route_of_few_and_of_all(pf, prec, accum32, n, r, sigma):
     f.run(_cuda(v.frames))
     _check_likelihoods(pf, f, prec, v.frames[-1], r, flags)
     f.close()
+
+
+@pytest.mark.parametrize("prec,accum32", [("f16", 0), ("f16", 1), ("bf16", 0)])
+@pytest.mark.parametrize("r", [5, 12, 14])
+@pytest.mark.parametrize("low", [0.0, -1.5, -6.0])
+def test_ancestors_of_tiles_with_row_sum_tables(pf, prec, accum32, r, low):
+    """The row sums of a tile's table lie in the memory of its strata counts and ancestor map: the
+    ancestors behind them are those of the CDF, in the first tile and in later ones, with the map's
+    first part in use, nearly all of it (low = -1.5: 7000 offspring of the first tile) and the counts
+    in its place (low = -6: more offspring than it holds)."""
+    v = synth.make_video(160, 140, 2, r, noise=8.0, seed=45, c0=(60.0, 60.0))
+    n = 9001
+    flags = pf.PF_FLAG_DEBUG_ARRAYS | (pf.PF_FLAG_ACCUM32 if accum32 else 0)
+    f = pf.Filter(v.W, v.H, n, r, prec, init=tuple(v.centres[0]), seed=46, flags=flags)
+    fr = _cuda(v.frames)
+    f.step(fr[0])
+    st = f.get_state()
+    st["L"] = np.where(np.arange(n) < 4096, 0.0, low)
+    st["max_l"], st["sum_e"] = 0.0, float(np.exp(st["L"]).sum())
+    f.set_state(st)
+    f.step(fr[1])
+    anc, c = f.debug(0).astype(np.int64), f.debug(1).astype(np.float64)
+    assert np.all(f.debug(2)[:, 2] > 0)
+    _check_likelihoods(pf, f, prec, v.frames[1], r, flags)
+    f.close()
+    assert np.array_equal(anc, oracle.resample(c, oracle.resample_u0(46, 0), "f32"))
