@@ -17,8 +17,9 @@ __device__ __forceinline__ int ancestor_tracker(const AncestorLaunch &G, int b) 
 }
 
 // Rejection: offspring per CTA of a tracker of n particles (a multiple of 32).  Small trackers are
-// spread over the SMs (kRejectionSpread CTAs, four an SM, while a CTA keeps 32 offspring, four a
-// warp): F32 1000 particles in one CTA of at most kRejectionOffspring 77 us a frame, so 13.
+// spread over the SMs (kRejectionSpread CTAs, four on each of the part's 152, while a CTA keeps 32
+// offspring): F32 1000 particles in one CTA of at most kRejectionOffspring 77 us a frame, so 14.
+// The host numbers the CTAs by the same function, so it depends on n alone.
 constexpr int kRejectionSpread = 608;
 __host__ __device__ inline int rejection_pool(int64_t n) {
     const int64_t p = ((n + kRejectionSpread - 1) / kRejectionSpread + 31) / 32 * 32;

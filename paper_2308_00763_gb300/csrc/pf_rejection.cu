@@ -18,13 +18,16 @@
 // threads share: each loop iteration is eight tries of every lane's current offspring (their
 // gathers in flight together), and a lane whose offspring is decided takes the next undecided
 // one from a shared counter, so a warp does not wait, for each group of 32 offspring, for the
-// largest of 32 geometric try counts.  Once the pool is empty the offspring still undecided
-// (one a thread at most) go to a list in shared memory, and each warp takes one at a time, 64
-// tries in order per iteration, two a lane: left to their own lanes, the last of a CTA's
-// offspring take as long as the whole pool before them.  Every offspring's tries and decision
-// are those of its own Philox stream either way.  Us a frame, 2048 a CTA without the list ->
-// rejection_pool(N) with it: F16 2^20 161 -> 129, 200003 91 -> 53, F32 30001 119 -> 28, BF16 5003
-// 119 -> 18, REF64 20003 100 -> 44.
+// largest of 32 geometric try counts.  Once the pool is empty, an offspring that its lane's eight
+// tries leave undecided (one a thread at most) goes to a list in shared memory, and each warp takes
+// one at a time, 64 tries in order per iteration, two a lane: left to their own lanes, the last of
+// a CTA's offspring take as long as the whole pool before them.  Every lane makes its eight tries
+// first, whatever the pool: over flat weights (the object lost) they decide every offspring, and a
+// warp's 64 for each were eight times the work.  Every offspring's tries and decision are those of
+// its own Philox stream either way.  Us a frame, 2048 a CTA without the list -> rejection_pool(N)
+// with it, on a tracked object: F16 2^20 161 -> 125, 200003 91 -> 51, F32 30001 119 -> 28, BF16 5003
+// 119 -> 19, REF64 20003 100 -> 44; over flat weights F16 2^20 54 -> 44, 150001 31 -> 20 (without
+// the lanes' own tries 70 and 51), sixteen trackers of 150001 133 -> 103 (487).
 #include <math.h>
 
 #include "pf_ancestor.cuh"
@@ -64,7 +67,7 @@ __global__ void __launch_bounds__(kRejectionThreads) rejection_kernel(const Ance
 
     int e = static_cast<int>(threadIdx.x);   // the lane's offspring (pool index); >= pool: none
     int i = 0;                               // its next try (a multiple of 8)
-    while (e < pool && *const_cast<volatile unsigned int *>(&s_next) < static_cast<unsigned int>(pool)) {
+    while (e < pool) {
         const int jj = static_cast<int>(j0) + e;
         const uint32_t tag = 6u + (static_cast<uint32_t>(jj) << 8);
         // eight tries at a time: proposals (four Philox blocks) and gathers first, all eight
@@ -98,6 +101,7 @@ __global__ void __launch_bounds__(kRejectionThreads) rejection_kernel(const Ance
             i = 0;
         } else {
             i += 8;
+            if (*const_cast<volatile unsigned int *>(&s_next) >= static_cast<unsigned int>(pool)) break;
         }
     }
     if (e < pool) {

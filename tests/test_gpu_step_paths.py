@@ -235,3 +235,15 @@ def test_ancestors_of_tiles_with_row_sum_tables(pf, prec, accum32, r, low):
     _check_likelihoods(pf, f, prec, v.frames[1], r, flags)
     f.close()
     assert np.array_equal(anc, oracle.resample(c, oracle.resample_u0(46, 0), "f32"))
+
+
+@pytest.mark.parametrize("prec,n", [("f32", 31), ("f16", 5003), ("bf16", 150001), ("ref64", 2047), ("f16", 200003)])
+def test_rejection_over_flat_weights(pf, prec, n):
+    """Equal weights accept the first try, which is the offspring's own index."""
+    frames = _cuda(np.full((2, 64, 64), 100, np.uint8))
+    f = pf.Filter(64, 64, n, 3, prec, init=(32.0, 32.0), seed=47, flags=pf.PF_FLAG_DEBUG_ARRAYS, resampler="rejection")
+    f.step(frames[0])
+    f.step(frames[1])
+    anc = f.debug(0)
+    f.close()
+    assert np.array_equal(anc, np.arange(n))
