@@ -1,8 +1,7 @@
 // pf_step.cu -- the fused per-frame SIR step for sm_103a.
 //
 // One launch per frame for a whole batch of trackers.  A tile is kTile consecutive
-// particles k of one tracker's previous frame.  Per tile (in ticket order; a CTA's first ticket
-// is its index):
+// particles k of one tracker's previous frame.  Per tile (in ticket order):
 //   1. resampling of the previous frame (Sec. IV, "Normalizing" and "Resampling"):
 //      e_k = exp(L_k - M) (Eq. 5 with the max of the previous step), a block scan, and a
 //      decoupled lookback over the tracker's earlier tiles give the inclusive prefix
@@ -2252,7 +2251,9 @@ template <int P> struct MinBlocks {
     static constexpr int value = (P == 0 ? 512 : 1024) / kThreads > 0 ? (P == 0 ? 512 : 1024) / kThreads : 1;
 };
 
-template <int P, int kMode>
+// kWaves: the launch may have more tiles than CTAs.  (Without the loop over tiles the step mode holds
+// its registers better: F16 2^20 particles 19.66 -> 19.10 us a frame, F32 600001 17.1 -> 16.8.)
+template <int P, int kMode, bool kWaves>
 __global__ void __launch_bounds__(kThreads, MinBlocks<P>::value) step_kernel(const StepLaunch Lp) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     StepSmem<P> &sm = *reinterpret_cast<StepSmem<P> *>(smem_raw);
@@ -2266,41 +2267,42 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<P>::value) step_kernel(con
     // without the programmatic-serialization attribute.)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (threadIdx.x == 0) sm.cached = Lp.ntrk == 1 ? 0 : -1;
+    // Tiles in ticket order, every ticket drawn: a tile waits for its predecessors (the lookback; the
+    // last tile's wait for all partials), and a drawn ticket says that the CTAs of all lower ones are
+    // running.  A CTA's index does not: CUDA promises no order of dispatch, and where fewer
+    // than gridDim.x CTAs are resident (a partition of the SMs, other kernels on them) the CTAs
+    // of a launch of several waves came back for tiles whose predecessors were first tiles of CTAs
+    // without an SM, and waited out their limit.  A launch of one wave draws once a CTA, while the
+    // state loads, and the last draw sets the word back (against CTA indices and no draw: F16 2^20
+    // particles 18.9 -> 19.1 us a frame, F32 21.6 -> 21.2, 600001 16.65 -> 16.8); a single tile waits
+    // for no other and draws none.  In a longer launch a ticket is drawn when the CTA is ready for
+    // it: drawn a tile ahead, its aggregate reaches the tiles that look back to it a tile later
+    // (2^24 F16 265 -> 329 us).
+    const auto total = [&] { return static_cast<uint32_t>(Lp.total_tiles); };
+    if (threadIdx.x == 0) {
+        uint32_t g = 0u;
+        if (total() > 1u) {
+            g = atomicAdd(Lp.ticket, 1u);
+            if (total() <= gridDim.x && g == total() - 1u) atomicExch(Lp.ticket, 0u);
+        }
+        sm.ticket = g;
+        sm.cached = Lp.ntrk == 1 ? 0 : -1;
+    }
     if (Lp.ntrk == 1) load_descriptor(Lp, Lp.slot_of ? __ldg(&Lp.slot_of[0]) : 0, 0, sm, Lp.preload ? 2 : 3);
     __syncthreads();
-    // Tiles in ticket order.  Where a launch can be a single wave, CTA b's first ticket is b (CTAs
-    // are dispatched in index order, so a tile's predecessors belong to running CTAs) and a
-    // launch of one wave draws none at all: a frame paid a draw before its tile and one to find
-    // none left, about 0.8 us each (with the descriptor load moved before the wait as well, F16
-    // frame at 2^20 particles 23.2 -> 22.1 us, 1000 particles F32 14.9 -> 12.7).  In a longer
-    // launch a ticket is drawn when the CTA is ready for it: drawn a tile ahead, its aggregate
-    // reaches the tiles that look back to it a tile later (2^24 F16 265 -> 329 us).
-    const uint32_t total = static_cast<uint32_t>(Lp.total_tiles);
-    if constexpr (kMode != kModeStepBig) {
-        // every CTA draws once for each tile it ran: total_tiles draws in all
-        for (uint32_t g = blockIdx.x; g < total;) {
+    if constexpr (kWaves) {
+        for (uint32_t g = sm.ticket; g < total();) {
             run_tile<P, kMode>(Lp, static_cast<int>(g), sm);
-            if (total <= gridDim.x) return;
+            if (total() <= gridDim.x) return;
             __syncthreads();
-            if (threadIdx.x == 0) sm.ticket = gridDim.x + atomicAdd(Lp.ticket, 1u);
-            __syncthreads();
-            g = sm.ticket;
-            if (threadIdx.x == 0 && g == gridDim.x + total - 1u) atomicExch(Lp.ticket, 0u);
-        }
-    } else {   // two waves or more (the loop above takes 28 more bytes of spills here, 2.6 % of the frame)
-        for (;;) {
             if (threadIdx.x == 0) sm.ticket = atomicAdd(Lp.ticket, 1u);
             __syncthreads();
-            const uint32_t g = sm.ticket;
-            __syncthreads();
-            if (g >= total) {
-                if (threadIdx.x == 0 && g == total + gridDim.x - 1u) atomicExch(Lp.ticket, 0u);
-                return;
-            }
-            run_tile<P, kMode>(Lp, static_cast<int>(g), sm);
-            __syncthreads();
+            g = sm.ticket;
         }
+        // (several waves: total_tiles + gridDim.x draws in all)
+        if (threadIdx.x == 0 && sm.ticket == total() + gridDim.x - 1u) atomicExch(Lp.ticket, 0u);
+    } else {
+        run_tile<P, kMode>(Lp, static_cast<int>(sm.ticket), sm);
     }
 }
 
@@ -2324,15 +2326,17 @@ int configure_and_grid(int total_tiles) {
                   "shared memory of the step kernel exceeds its CTAs per SM");
     if (sizeof(StepSmem<P>) + 1024 > 228 * 1024) return -1;
     const int bytes = static_cast<int>(sizeof(StepSmem<P>));
-    if (cudaFuncSetAttribute(step_kernel<P, kModeStep>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-        cudaFuncSetAttribute(step_kernel<P, kModeStepBig>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-        cudaFuncSetAttribute(step_kernel<P, kModeCdf>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-        cudaFuncSetAttribute(step_kernel<P, kModePull>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess)
+    const auto allow = [&](auto *k) {
+        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+    };
+    if (!allow(step_kernel<P, kModeStep, false>) || !allow(step_kernel<P, kModeStep, true>) ||
+        !allow(step_kernel<P, kModeStepBig, true>) || !allow(step_kernel<P, kModeCdf, true>) ||
+        !allow(step_kernel<P, kModePull, true>))
         return -1;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_kernel<P, kModeStep>, kThreads, bytes);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_kernel<P, kModeStep, false>, kThreads, bytes);
     if (per_sm < 1) per_sm = 1;
     const int g = sms * per_sm;
     return total_tiles < g ? total_tiles : g;
@@ -2399,7 +2403,7 @@ int step_grid_size(int precision, int total_tiles) {
 // the stream is a step kernel (the previous frame), this launch is scheduled while that one
 // drains and waits for it on the device (griddepcontrol.wait) instead of the stream
 // serialising the two; captured into a CUDA graph as a programmatic dependency.
-template <int P, int kMode>
+template <int P, int kMode, bool kWaves>
 int launch_one(int grid, const StepLaunch &L, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
@@ -2411,19 +2415,20 @@ int launch_one(int grid, const StepLaunch &L, cudaStream_t s) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return static_cast<int>(cudaLaunchKernelEx(&cfg, step_kernel<P, kMode>, L));
+    return static_cast<int>(cudaLaunchKernelEx(&cfg, step_kernel<P, kMode, kWaves>, L));
 }
 
-template <int kMode>
+template <int kMode, bool kWaves = true>
 int launch_mode(int precision, const StepLaunch &L, int grid, void *stream) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (grid < 1) grid = 1;
+    if (L.total_tiles < 1) return 0;
+    grid = std::max(1, std::min(grid, static_cast<int>(L.total_tiles)));   // (one wave: a CTA a tile)
     int rc = -1;
     switch (precision) {
-        case 0: rc = launch_one<0, kMode>(grid, L, s); break;
-        case 1: rc = launch_one<1, kMode>(grid, L, s); break;
-        case 2: rc = launch_one<2, kMode>(grid, L, s); break;
-        case 3: rc = launch_one<3, kMode>(grid, L, s); break;
+        case 0: rc = launch_one<0, kMode, kWaves>(grid, L, s); break;
+        case 1: rc = launch_one<1, kMode, kWaves>(grid, L, s); break;
+        case 2: rc = launch_one<2, kMode, kWaves>(grid, L, s); break;
+        case 3: rc = launch_one<3, kMode, kWaves>(grid, L, s); break;
         default: return -1;
     }
     if (rc != 0) return rc;
@@ -2434,6 +2439,7 @@ int launch_step(int precision, const StepLaunch &L, int grid, void *stream) {
     // a single tracker of at least two waves of tiles takes the instantiation with the
     // tracker table (the kernel checks the condition again per tile)
     if (L.ntrk == 1 && L.total_tiles >= 2 * grid) return launch_mode<kModeStepBig>(precision, L, grid, stream);
+    if (L.total_tiles <= std::max(1, grid)) return launch_mode<kModeStep, false>(precision, L, grid, stream);
     return launch_mode<kModeStep>(precision, L, grid, stream);
 }
 
