@@ -819,10 +819,15 @@ class Server:
         if on_dev:
             q[1].append((q[0], keep))
         q[0] += 1
-        if len(q[1]) > 2 * self.cfg.queue_depth:   # (at most queue_depth are still in use)
-            done = pf_server_frames_done(self.h, sid)
-            q[1] = [(i, t) for i, t in q[1] if i >= done]
+        if len(q[1]) > 1:   # (an older one; host frames are copied and none is held)
+            self._drop(q[1], pf_server_frames_done(self.h, sid))
         return True
+
+    @staticmethod
+    def _drop(held, done):
+        """Let go of the frames before number `done`."""
+        while held and held[0][0] < done:
+            held.pop(0)
 
     def tick(self):
         return pf_server_tick(self.h)
@@ -831,7 +836,10 @@ class Server:
         return pf_server_poll(self.h)
 
     def drain(self):
+        held = [(q[1], q[0]) for q in self._keep.values() if q[1]]
         pf_server_drain(self.h)
+        for frames, submitted in held:   # (whatever was submitted before the call)
+            self._drop(frames, submitted)
 
     def result(self, sid, index):
         rc, xy = pf_server_result(self.h, sid, index)
