@@ -247,3 +247,37 @@ def test_rejection_over_flat_weights(pf, prec, n):
     anc = f.debug(0)
     f.close()
     assert np.array_equal(anc, np.arange(n))
+
+
+@pytest.mark.parametrize("prec,accum32", [("f16", 0), ("f16", 1), ("bf16", 0)])
+@pytest.mark.parametrize("r", [5, 10, 14, 16])
+@pytest.mark.parametrize("resampler", ["systematic", "multinomial", "metropolis", "rejection"])
+def test_production_tables_by_row_sums(pf, prec, accum32, r, resampler):
+    """Trackers without debug arrays: the pull kernel's row sums lie over the ancestor map (debug arrays
+    keep it in use, and the sums away), in one band up to radius 10 in F16 and in several beyond; the
+    step kernel's pairs take their fast copy.  A second tracker with debug arrays has a table in
+    every tile, and the same particles."""
+    v = synth.make_video(160, 140, 3, r, noise=8.0, seed=48, c0=(60.0, 60.0))
+    flags = pf.PF_FLAG_ACCUM32 if accum32 else 0
+    states = []
+    for debug in (0, pf.PF_FLAG_DEBUG_ARRAYS):
+        f = pf.Filter(v.W, v.H, 3001, r, prec, init=tuple(v.centres[0]), seed=49, flags=flags | debug, resampler=resampler)
+        f.run(_cuda(v.frames))
+        _check_likelihoods(pf, f, prec, v.frames[-1], r, flags)
+        states.append(f.get_state())
+        if debug:
+            assert np.all(f.debug(2)[:, 2] > 0)
+        f.close()
+    for k in ("x", "y", "L", "est_x", "est_y", "sum_e"):
+        assert np.array_equal(states[0][k], states[1][k])
+
+
+@pytest.mark.parametrize("prec", ["ref64", "f32", "f16", "bf16"])
+@pytest.mark.parametrize("resampler", ["multinomial", "metropolis"])
+@pytest.mark.parametrize("n,sigma", [(40001, (5.0, 2.0)), (3001, (40.0, 40.0))])
+def test_direct_route_of_the_pull_kernel(pf, prec, resampler, n, sigma):
+    v = synth.make_video(200, 150, 3, 6, noise=8.0, seed=50)
+    f = pf.Filter(v.W, v.H, n, 5, prec, init=tuple(v.centres[0]), seed=51, sigma=sigma, resampler=resampler)
+    f.run(_cuda(v.frames))
+    _check_likelihoods(pf, f, prec, v.frames[-1], 5)
+    f.close()
