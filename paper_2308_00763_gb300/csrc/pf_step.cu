@@ -1198,6 +1198,8 @@ __device__ __forceinline__ void table_by_rows(StepSmem<P> &sm, int rw, int pw, i
     const TrackerDev &T = sm.trk;
     const int r = T.r, ncls = T.ncls, tid = threadIdx.x;
     R *rows = reinterpret_cast<R *>(row_words<P, kMode>(sm, words));
+    const int cap = kMode != kModeStep ? kMapMax / 2 : (words > kTile ? kRowWords : kTile);   // words from there on
+    (void)cap;
     const auto zero = [] { if constexpr (kPair) return __float2half2_rn(0.0f); else return 0.0f; };
     const auto add = [](R a, R b) { if constexpr (kPair) return __hadd2(a, b); else return a + b; };
     const auto term = [&](int i) {
@@ -1221,11 +1223,11 @@ __device__ __forceinline__ void table_by_rows(StepSmem<P> &sm, int rw, int pw, i
                     if (ad <= h2) a2 = add(a2, t);
                     if (ad <= h3) a3 = add(a3, t);
                 }
-                R *o = rows + (c * nr + yy) * pw + hp;
-                o[0] = a0;
-                if (h1 >= 0) o[nr * pw] = a1;
-                if (h2 >= 0) o[2 * nr * pw] = a2;
-                if (h3 >= 0) o[3 * nr * pw] = a3;
+                const int o = (c * nr + yy) * pw + hp;
+                rows[PF_IDX(o, cap)] = a0;
+                if (h1 >= 0) rows[PF_IDX(o + nr * pw, cap)] = a1;
+                if (h2 >= 0) rows[PF_IDX(o + 2 * nr * pw, cap)] = a2;
+                if (h3 >= 0) rows[PF_IDX(o + 3 * nr * pw, cap)] = a3;
             }
         }
         __syncthreads();
@@ -1233,7 +1235,7 @@ __device__ __forceinline__ void table_by_rows(StepSmem<P> &sm, int rw, int pw, i
             const int cy = i / pw, hp = i - cy * pw;
             R acc = zero();
 #pragma unroll 4
-            for (int k = 0; k <= 2 * r; ++k) acc = add(acc, rows[PF_IDX((T.rc[k] * nr + cy + k) * pw + hp, kRowWords)]);
+            for (int k = 0; k <= 2 * r; ++k) acc = add(acc, rows[PF_IDX((T.rc[k] * nr + cy + k) * pw + hp, cap)]);
             if constexpr (kPair) {
                 const int cx = 2 * hp, c = (y0 + cy) * ww + cx;
                 sm.table[PF_IDX(c, kTableMax)] = __low2half(acc);
@@ -1269,7 +1271,7 @@ __device__ __forceinline__ void cdf_search(const TrackerDev &T, const typename P
     A *cs = reinterpret_cast<A *>(&sm);
     for (int i = threadIdx.x; i < nb; i += kThreads) {
         const int64_t last = ((static_cast<int64_t>(i) + 1) << lb) - 1;
-        cs[i] = __ldg(c64 + (last < n64 ? last : n64 - 1));
+        cs[PF_IDX(i, kCoarse)] = __ldg(c64 + (last < n64 ? last : n64 - 1));
     }
     __syncthreads();
 #pragma unroll
@@ -1278,7 +1280,7 @@ __device__ __forceinline__ void cdf_search(const TrackerDev &T, const typename P
 #pragma unroll
         for (int m = 0; m < kItems; ++m) {
             const int q = k[m] + w;
-            if (q <= nb && !(cs[q - 1] >= u[m])) k[m] = q;
+            if (q <= nb && !(cs[PF_IDX(q - 1, kCoarse)] >= u[m])) k[m] = q;
         }
     }
     __syncthreads();                      // (the memory of cs is the tile's again)
@@ -1288,18 +1290,20 @@ __device__ __forceinline__ void cdf_search(const TrackerDev &T, const typename P
 #pragma unroll
         for (int m = 0; m < kItems; ++m) {
             const int q = k[m] + w;
-            if (q <= n8 && !(__ldg(c8 + q - 1) >= u[m])) k[m] = q;
+            if (q <= n8 && !(__ldg(c8 + PF_IDX(q - 1, n8)) >= u[m])) k[m] = q;
         }
     }
-    // entries below u among c[k .. k + 8), n of them in all
+    // entries below u among c[k .. k + 8), n of them in all and room for a whole number of eights
     const auto count8 = [&](const A *c, int n) {
+        const int starts = ((n + 7) & ~7) - 7;
+        (void)starts;
 #pragma unroll
         for (int g = 0; g < kItems; g += 4) {
             uint4 v[4][8 / kVec];
 #pragma unroll
             for (int m = 0; m < 4; ++m)
 #pragma unroll
-                for (int i = 0; i < 8 / kVec; ++i) v[m][i] = __ldg(reinterpret_cast<const uint4 *>(c + k[g + m]) + i);
+                for (int i = 0; i < 8 / kVec; ++i) v[m][i] = __ldg(reinterpret_cast<const uint4 *>(c + PF_IDX(k[g + m], starts)) + i);
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
                 int below = 0;

@@ -249,3 +249,42 @@ def test_thread_block_study_builds_keep_the_method(threads):
     assert ("/t%d/" % threads) in out["lib"]
     for prec, N, exact, monotone, ok, err in out["cases"]:
         assert exact and monotone and ok, (threads, prec, N, err)
+
+
+ROWS_CHILD = r'''
+import sys
+sys.path.insert(0, sys.argv[1])
+import numpy as np, torch
+import paper_2308_00763_gb300 as pf
+from paper_2308_00763_gb300 import synth
+pf.lib(build_if_missing=True)
+assert "/checked/" in pf.library_path()
+for r in (5, 14, 16):
+    v = synth.make_video(160, 140, 3, r, noise=8.0, seed=48, c0=(60.0, 60.0))
+    for prec, flags in (("f16", 0), ("f16", pf.PF_FLAG_ACCUM32), ("bf16", 0)):
+        for res in ("systematic", "multinomial"):
+            f = pf.Filter(v.W, v.H, 9001, r, prec, init=tuple(v.centres[0]), seed=49, flags=flags, resampler=res)
+            f.run(torch.from_numpy(v.frames).cuda())
+            assert np.all(np.isfinite(f.estimates(0, v.T)))   # (an index out of range fails the step)
+            f.close()
+v = synth.make_video(128, 128, 3, 5, noise=5.0, seed=25)
+for prec, n in (("f32", 7), ("f32", 4097), ("f32", (1 << 20) + 9), ("ref64", 700001), ("f16", 3000001)):
+    f = pf.Filter(v.W, v.H, n, 5, prec, init=tuple(v.centres[0]), seed=26, resampler="multinomial")
+    f.run(torch.from_numpy(v.frames).cuda())
+    assert np.all(np.isfinite(f.estimates(0, v.T)))
+    f.close()
+print("clean")
+'''
+
+
+def test_checked_build_covers_row_sums_and_the_multinomial_search():
+    """Production trackers (no debug arrays): the row sums' places in the step and the pull kernel, and
+    the three levels of the search, which read whole groups of eight."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    env = dict(os.environ, PF_CHECKED="1")
+    env.pop("PF_STEP_THREADS", None)
+    env.pop("PF_NAIVE", None)
+    p = subprocess.run([sys.executable, "-c", ROWS_CHILD, ROOT], env=env, capture_output=True, text=True, timeout=900)
+    assert p.returncode == 0 and "clean" in p.stdout, (p.stdout[-2000:], p.stderr[-4000:])
