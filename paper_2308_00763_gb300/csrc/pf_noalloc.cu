@@ -9,6 +9,7 @@
 // decoupled-lookback descriptors, per-tile partial sums, counters and the tracker's
 // descriptor) lives here, in a file-scope device array that exists in every GPU's memory
 // as soon as the library is loaded and stays there until the process exits.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stddef.h>
@@ -32,7 +33,7 @@ constexpr int kMaxDevices = 64;
 constexpr size_t kScratchBytes = 8192 + (sizeof(LookbackDesc) + sizeof(TilePartial)) * size_t(kMaxTiles);
 
 // The scratch array.  In host code its name is only a stand-in for the symbol; the
-// device address comes from cudaGetSymbolAddress (per device).
+// device address comes from cudaGetSymbolAddress (per context).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 // Layout inside the scratch array.
@@ -99,26 +100,68 @@ bool overlaps(const void *a, const void *b, size_t n) {
     return x < y + n && y < x + n;
 }
 
+// What a call needs looked up.  The scratch array is a device variable, of which every context has
+// its own copy at its own address, and the step kernels' shared-memory limits are a context's
+// as well; a context is known by its id, which the driver never gives out twice.
+struct ContextEntry {
+    unsigned long long id;
+    unsigned char *scratch;   // null: the entry is free
+    int grid[4];
+};
 std::mutex g_lock;
-unsigned char *g_scratch_dev[kMaxDevices] = {};
-int g_grid[kMaxDevices][4] = {};
+ContextEntry g_ctx[16] = {};   // (more contexts than this take turns and are looked up again)
+int g_ctx_next = 0;
 
-// Device address of the scratch array on the current device (looked up once per device).
-pf_status scratch_for_current_device(int *dev_out, unsigned char **ptr_out) {
+bool current_context_id(unsigned long long *id) {
+    using GetId = CUresult (*)(CUcontext, unsigned long long *);
+    static const GetId get = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<GetId>(f);
+    }();
+    return get && get(nullptr, id) == CUDA_SUCCESS;
+}
+
+// Address of the scratch array in the current context and the step's grid there.
+pf_status scratch_for_current_context(int precision, unsigned char **ptr_out, int *grid_out) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return PF_ERR_CUDA; }
     if (dev < 0 || dev >= kMaxDevices) return PF_ERR_ARG;
     std::lock_guard<std::mutex> guard(g_lock);
-    if (!g_scratch_dev[dev]) {
+    ContextEntry *e = nullptr, unknown = {};
+    unsigned long long id = 0;
+    if (!current_context_id(&id)) {
+        e = &unknown;   // (looked up on every call)
+    } else {
+        for (ContextEntry &c : g_ctx)
+            if (c.scratch && c.id == id) e = &c;
+        if (!e) {
+            e = &g_ctx[g_ctx_next];
+            g_ctx_next = (g_ctx_next + 1) % static_cast<int>(sizeof(g_ctx) / sizeof(g_ctx[0]));
+            *e = ContextEntry{};
+            e->id = id;
+        }
+    }
+    if (!e->scratch) {
         void *p = nullptr;
         if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) {
             cudaGetLastError();
             return PF_ERR_CUDA;
         }
-        g_scratch_dev[dev] = static_cast<unsigned char *>(p);
+        e->scratch = static_cast<unsigned char *>(p);
     }
-    *dev_out = dev;
-    *ptr_out = g_scratch_dev[dev];
+    if (!e->grid[precision]) {
+        const int g = step_grid_size(precision, kMaxTiles);
+        if (g < 1) return PF_ERR_CUDA;
+        e->grid[precision] = g;
+    }
+    *ptr_out = e->scratch;
+    *grid_out = e->grid[precision];
     return PF_OK;
 }
 
@@ -168,9 +211,9 @@ extern "C" pf_status pf_step_frame_noalloc(const pf_config *cfg, const pf_state_
         if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess) { cudaGetLastError(); return PF_ERR_CUDA; }
         if (cs != cudaStreamCaptureStatusNone) return PF_ERR_ARG;
     }
-    int dev = 0;
     unsigned char *scr = nullptr;
-    pf_status s = scratch_for_current_device(&dev, &scr);
+    int grid = 0;
+    pf_status s = scratch_for_current_context(c.precision, &scr, &grid);
     if (s != PF_OK) return s;
     constexpr ScratchLayout LY = layout();
 
@@ -222,13 +265,6 @@ extern "C" pf_status pf_step_frame_noalloc(const pf_config *cfg, const pf_state_
     noalloc_setup_kernel<<<8, 256, 0, stream>>>(sp, scr, nt);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return PF_ERR_CUDA;
-    int grid;
-    {
-        std::lock_guard<std::mutex> guard(g_lock);
-        if (!g_grid[dev][c.precision]) g_grid[dev][c.precision] = step_grid_size(c.precision, kMaxTiles);
-        grid = g_grid[dev][c.precision];
-    }
-    if (grid < 1) return PF_ERR_CUDA;
     if (grid > nt) grid = nt;
     StepLaunch L;
     L.trk = reinterpret_cast<const TrackerDev *>(scr + LY.trk);

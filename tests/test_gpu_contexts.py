@@ -62,6 +62,42 @@ def run_engine(prec):
     same(first, engine(prec))     # (and the first context is as it was)
 
 
+def noalloc(prec):   # two frames through the allocation-free entry point, in the current context
+    n, size = 5001, {"ref64": 8, "f32": 4, "f16": 2}[prec]
+
+    def alloc(nbytes):
+        p = ctypes.c_uint64()
+        check(cu.cuMemAlloc_v2(ctypes.byref(p), ctypes.c_size_t(nbytes)), "cuMemAlloc")
+        return p.value
+
+    frames = alloc(v.frames[:2].nbytes)
+    host = np.ascontiguousarray(v.frames[:2])
+    check(cu.cuMemcpyHtoD_v2(ctypes.c_uint64(frames), host.ctypes.data_as(ctypes.c_void_p), ctypes.c_size_t(host.nbytes)),
+          "cuMemcpyHtoD")
+    slots = [[alloc(n * size) for _ in range(3)] for _ in range(2)]
+    cfg = pf.make_config(v.W, v.H, n, 4, prec, init=tuple(v.centres[0]), seed=53)
+    hdr = pf.PfStateHeader(magic=0x31534650, precision=cfg.precision, num_particles=n, t=0)
+    step = host.strides[0]
+    hdr = pf.pf_step_frame_noalloc(cfg, hdr, 0, 0, 0, frames, v.W, *slots[0], stream=0)
+    hdr = pf.pf_step_frame_noalloc(cfg, hdr, *slots[0], frames + step, v.W, *slots[1], stream=0)
+    out = [np.frombuffer(bytes(hdr), np.uint8)]
+    for p in slots[1]:
+        a = np.empty(n * size, np.uint8)
+        check(cu.cuMemcpyDtoH_v2(a.ctypes.data_as(ctypes.c_void_p), ctypes.c_uint64(p), ctypes.c_size_t(a.nbytes)),
+              "cuMemcpyDtoH")
+        out.append(a)
+    for p in [frames] + slots[0] + slots[1]:
+        check(cu.cuMemFree_v2(ctypes.c_uint64(p)), "cuMemFree")
+    return out
+
+
+def run_noalloc(prec):
+    engine(prec)                  # (the first context is the library's own choice)
+    first = noalloc(prec)
+    same(first, in_second_context(lambda: noalloc(prec)))
+    same(first, noalloc(prec))
+
+
 globals()["run_" + sys.argv[1]](sys.argv[2])
 print("same bits")
 """
@@ -80,3 +116,11 @@ def test_filter_in_a_second_context(prec):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     _child("engine", prec)
+
+
+@pytest.mark.parametrize("prec", ["ref64", "f32", "f16"])
+def test_allocation_free_step_in_a_second_context(prec):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    _child("noalloc", prec)
