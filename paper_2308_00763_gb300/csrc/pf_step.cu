@@ -790,9 +790,9 @@ struct __align__(16) StepSmem {
     TrackerDev trk;
     TrackerState st;
     FrameRef fr;
-    alignas(16) uint16_t map[kMapMax];   // ancestor (tile element + 1) of each offspring
-    // last: only the step mode allocates it (see counts_array and row_words)
-    alignas(16) int32_t J[kTile];
+    // last: the strata counts and the ancestor map of the step mode, whose row sums lie over both;
+    // the other modes allocate the first half, their map (see counts_array)
+    alignas(16) int32_t tail[2 * kTile];
 };
 
 // Block-wide merge of per-thread stats, result valid in thread 0.  Each warp takes its
@@ -1155,24 +1155,28 @@ constexpr int kModeStepBig = 3;
 // searches run in (2^19 F16 50.8 us against 51.4).
 template <int P, int kMode>
 __device__ __forceinline__ int32_t *counts_array(StepSmem<P> &sm) {
-    return kMode == kModeStep ? sm.J : reinterpret_cast<int32_t *>(sm.map);
+    return sm.tail;
 }
-// Where the table's row sums lie while it is built.  In the step mode in J's memory, not written
-// before the table is read, and, if there are more, from the map's second half on, which is
+// Ancestor (tile element + 1) of each offspring.
+template <int P, int kMode>
+__device__ __forceinline__ uint16_t *map_array(StepSmem<P> &sm) {
+    return reinterpret_cast<uint16_t *>(kMode == kModeStep ? sm.tail + kTile : sm.tail);
+}
+// Where the table's row sums lie while it is built: in the step mode in the counts' memory, not
+// written before the table is read, and, if there are more, in the map's first half, which is
 // cleared again behind them.  (An array of their own, 24 KB more a CTA, left the L1 28 KB an SM of
 // 92: F16, noise 40, 65536 particles, radius 5, all scored from the frame, 297 us a frame against
-// 202; 2^20 722 against 456; the same at noise 1.)  In the pull mode the map, which has no use there
-// but for the ancestors' indices when debug arrays are on.
-template <int P, int kMode>
-__device__ __forceinline__ uint32_t *row_words(StepSmem<P> &sm, int words) {
-    static_assert(offsetof(StepSmem<P>, J) == offsetof(StepSmem<P>, map) + sizeof(sm.map), "the map's end and J are one piece");
-    uint32_t *const m = reinterpret_cast<uint32_t *>(sm.map);
-    return kMode != kModeStep ? m : m + kMapMax / 2 - (words > kTile ? kRowWords - kTile : 0);
+// 202; 2^20 722 against 456; the same at noise 1.  A place that starts where the number of words says
+// costs an address a load: BF16 300007 particles, radius 10, 17.0 against 16.6.)  In the pull
+// mode the map, which has no use there but for the ancestors' indices when debug arrays are on.
+template <int P>
+__device__ __forceinline__ uint32_t *row_words(StepSmem<P> &sm) {
+    return reinterpret_cast<uint32_t *>(sm.tail);
 }
 template <int P, int kMode> constexpr size_t smem_bytes() {
-    return kMode == kModeStep ? sizeof(StepSmem<P>) : offsetof(StepSmem<P>, J);
+    return kMode == kModeStep ? sizeof(StepSmem<P>) : offsetof(StepSmem<P>, tail) + sizeof(int32_t) * kTile;
 }
-static_assert(sizeof(uint16_t) * kMapMax == sizeof(int32_t) * kTile, "J fits the map's memory");
+static_assert(sizeof(uint16_t) * kMapMax == sizeof(int32_t) * kTile, "the map and the counts are of one size");
 
 // The half-form table of a window from the staged terms, by row sums.  A cell is the sum of its
 // template rows top to bottom, each summed left to right (HalfLik); a row's sum depends only on
@@ -1190,16 +1194,15 @@ static_assert(sizeof(uint16_t) * kMapMax == sizeof(int32_t) * kTile, "J fits the
 // particles r = 12 18.8 -> 16.1; F16 2^20 particles r = 5 21.8 -> 22.0 (there the tiles build
 // their tables while they wait for their predecessors).
 template <int P, int kMode, bool kPair>
-__device__ __forceinline__ void table_by_rows(StepSmem<P> &sm, int rw, int pw, int ww, int wh, int band, int words,
+__device__ __forceinline__ void table_by_rows(StepSmem<P> &sm, int rw, int pw, int ww, int wh, int band,
                                               TrackerState *st) {
     (void)st;
     using H = typename Prec<P>::pos_t;
     using R = typename std::conditional<kPair, __half2, float>::type;
     const TrackerDev &T = sm.trk;
     const int r = T.r, ncls = T.ncls, tid = threadIdx.x;
-    R *rows = reinterpret_cast<R *>(row_words<P, kMode>(sm, words));
-    const int cap = kMode != kModeStep ? kMapMax / 2 : (words > kTile ? kRowWords : kTile);   // words from there on
-    (void)cap;
+    R *rows = reinterpret_cast<R *>(row_words(sm));
+    constexpr int cap = kMode == kModeStep ? kRowWords : kMapMax / 2;   // words there
     const auto zero = [] { if constexpr (kPair) return __float2half2_rn(0.0f); else return 0.0f; };
     const auto add = [](R a, R b) { if constexpr (kPair) return __hadd2(a, b); else return a + b; };
     const auto term = [&](int i) {
@@ -1488,7 +1491,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
         // clear the ancestor map (its heads are written after the strata are counted)
 #pragma unroll
         for (int i = 0; i < kMapMax / 8 / kThreads; ++i)
-            reinterpret_cast<uint4 *>(sm.map)[tid + i * kThreads] = make_uint4(0u, 0u, 0u, 0u);
+            reinterpret_cast<uint4 *>(map_array<P, kMode>(sm))[tid + i * kThreads] = make_uint4(0u, 0u, 0u, 0u);
         const float sx = Tr::kHalf ? static_cast<float>(axi_anc) : 0.0f;
         const float sy = Tr::kHalf ? static_cast<float>(ayi_anc) : 0.0f;
         // FP64: a warp wholly past the tile's end (a REF64 tile may hold a quarter of kTile)
@@ -1764,17 +1767,16 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             by_rows = (paired || !hk.half_acc) && (band == wh || band >= 4) && by_row < by_cell &&
                       (kMode == kModeStep || (kMode == kModePull && !T.dbg_anc));
             if (by_rows) {
-                const int words = T.ncls * pw * (band + 2 * r);
                 if constexpr (P == 2) {
-                    if (paired) table_by_rows<P, kMode, true>(sm, rw, pw, ww, wh, band, words, st);
+                    if (paired) table_by_rows<P, kMode, true>(sm, rw, pw, ww, wh, band, st);
                 }
-                if (!paired) table_by_rows<P, kMode, false>(sm, rw, pw, ww, wh, band, words, st);
+                if (!paired) table_by_rows<P, kMode, false>(sm, rw, pw, ww, wh, band, st);
                 if constexpr (kMode == kModeStep) {
-                    if (words > kTile) {   // the map's second half was in use
+                    if (T.ncls * pw * (band + 2 * r) > kTile) {   // the map's first half was in use
                         __syncthreads();
-                        reinterpret_cast<uint4 *>(sm.map)[kThreads + tid] = make_uint4(0u, 0u, 0u, 0u);
+                        reinterpret_cast<uint4 *>(map_array<P, kMode>(sm))[tid] = make_uint4(0u, 0u, 0u, 0u);
                     }
-                    if (lt == 0) __syncthreads();   // (before J and the map are written; else the lookback's)
+                    if (lt == 0) __syncthreads();   // (before counts and map are written; else the lookback's)
                 }
             }
         }
@@ -1933,10 +1935,10 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
 #pragma unroll
                 for (int m = 0; m < kItems; ++m) {
                     if (Jr[m] > jp && jp - mbl < kMapMax)
-                        sm.map[PF_IDX(jp - mbl, kMapMax)] = static_cast<uint16_t>(eb + m + 1);
+                        map_array<P, kMode>(sm)[PF_IDX(jp - mbl, kMapMax)] = static_cast<uint16_t>(eb + m + 1);
                     jp = Jr[m];
                 }
-                if constexpr (kMode == kModeStep) store_items(sm.J + eb, Jr);
+                if constexpr (kMode == kModeStep) store_items(counts_array<P, kMode>(sm) + eb, Jr);
                 if (eb + kItems >= cnt) sm.jend = Jr[kItems - 1];   // the tile's last element's owner
             }
         }
@@ -1961,7 +1963,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
     if (use_map) {
         // thread tid fills entries [tid*ch, tid*ch + ch), ch = 8 or 16 (16-byte vectors)
         const int nv = (je - mb > kThreads * 8) ? 2 : 1;
-        uint4 *mv = reinterpret_cast<uint4 *>(sm.map) + tid * nv;
+        uint4 *mv = reinterpret_cast<uint4 *>(map_array<P, kMode>(sm)) + tid * nv;
         uint4 c0 = mv[0], c1 = make_uint4(0u, 0u, 0u, 0u);
         if (nv == 2) c1 = mv[1];
         uint32_t m2 = __vmaxu2(__vmaxu2(__vmaxu2(c0.x, c0.y), __vmaxu2(c0.z, c0.w)),
@@ -2033,7 +2035,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
         const int j0 = 2 * q, j1 = j0 + 1;
         int e0 = 0, e1 = 0;
         if (kFast) {
-            const uint32_t mw = reinterpret_cast<const uint32_t *>(sm.map)[PF_IDX(q - (mb >> 1), kMapMax / 2)];
+            const uint32_t mw = reinterpret_cast<const uint32_t *>(map_array<P, kMode>(sm))[PF_IDX(q - (mb >> 1), kMapMax / 2)];
             e0 = static_cast<int>(mw & 0xffffu) - 1;
             e1 = static_cast<int>(mw >> 16) - 1;
         } else if (t > 0) {
@@ -2043,8 +2045,8 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
                 e0 = j0 - k0;
                 e1 = j1 - k0;
             } else if (use_map) {
-                e0 = v0 ? static_cast<int>(sm.map[PF_IDX(j0 - mb, kMapMax)]) - 1 : 0;
-                e1 = v1 ? static_cast<int>(sm.map[PF_IDX(j1 - mb, kMapMax)]) - 1 : 0;
+                e0 = v0 ? static_cast<int>(map_array<P, kMode>(sm)[PF_IDX(j0 - mb, kMapMax)]) - 1 : 0;
+                e1 = v1 ? static_cast<int>(map_array<P, kMode>(sm)[PF_IDX(j1 - mb, kMapMax)]) - 1 : 0;
             } else {
                 if (v0) e0 = upper_index(counts_array<P, kMode>(sm), cnt, j0);
                 if (v1) e1 = (v0 && counts_array<P, kMode>(sm)[e0] > j1) ? e0 : upper_index(counts_array<P, kMode>(sm), cnt, j1);
