@@ -211,7 +211,7 @@ constexpr int kGumbelOffspring = 8;       // Gumbel-max: offspring per CTA
 constexpr int kGumbelThreads = 256;
 constexpr int kMetropolisThreads = 256;   // Metropolis: one offspring per thread
 constexpr int kRejectionThreads = 256;    // rejection: threads per CTA
-constexpr int kRejectionOffspring = 2048; // rejection: offspring per CTA (a pool its threads share)
+constexpr int kRejectionOffspring = 2048; // rejection: most offspring a CTA (its threads share a pool; rejection_pool)
 struct AncestorLaunch {
     const TrackerDev *trk;     // device array indexed by slot
     const FrameRef *frames;    // device array indexed by slot

@@ -27,7 +27,9 @@ using namespace pfk;
 namespace {
 
 constexpr int64_t kMaxParticles = int64_t(1) << 22;
-constexpr int kMaxTiles = static_cast<int>(kMaxParticles / (kTile / 2));   // a tile holds >= kTile / 2
+// A tile holds kTile / 2 particles or more, but for the smaller tiles of a REF64 tracker, which number
+// at most one a resident CTA (step_tile_size); a call whose tiles are more is refused.
+constexpr int kMaxTiles = static_cast<int>(kMaxParticles / (kTile / 2));
 constexpr int kMaxDevices = 64;
 // tracker descriptor, state, frame and counters, then the per-tile descriptors and partials
 constexpr size_t kScratchBytes = 8192 + (sizeof(LookbackDesc) + sizeof(TilePartial)) * size_t(kMaxTiles);

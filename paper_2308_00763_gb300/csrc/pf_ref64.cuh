@@ -17,7 +17,8 @@
 //   radius        0.852 (0.3254) -> 0.852 (0.3254)
 //   sine, cosine  1.476 (0.3610) -> 1.093 (0.2888)
 //   exponential   0.888 (0.3017) -> 0.501 (0.2887)
-// Measured us a frame, library functions -> tables: 2^20 particles 375 -> 227, 200003 231 -> 134.
+// Measured us a frame when they came in, library functions -> tables: 2^20 particles 375 -> 227, 200003
+// 231 -> 134 (the sine and cosine as accurate as above: 2 % of the step now).
 #pragma once
 #include <stdint.h>
 

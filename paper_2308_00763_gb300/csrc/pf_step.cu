@@ -1191,8 +1191,7 @@ static_assert(sizeof(uint16_t) * kMapMax == sizeof(int32_t) * kTile, "the map an
 // idle in a chain of |D| dependent additions.  Windows whose row sums do not fit are done in
 // bands of `band` cell rows.  Measured us a
 // frame, cells one by one -> row sums: BF16 300007 particles r = 10 20.9 -> 19.0, F16 4096
-// particles r = 12 18.8 -> 16.1; F16 2^20 particles r = 5 21.8 -> 22.0 (there the tiles build
-// their tables while they wait for their predecessors).
+// particles r = 12 18.8 -> 16.1; r = 5, F16 2^20 particles 19.4 -> 18.9, 450001 15.8 -> 15.0.
 template <int P, int kMode, bool kPair>
 __device__ __forceinline__ void table_by_rows(StepSmem<P> &sm, int rw, int pw, int ww, int wh, int band,
                                               TrackerState *st) {
@@ -2097,7 +2096,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             const bool in1 = cx1 < static_cast<unsigned>(ww) && cy1 < static_cast<unsigned>(wh);
             acc_t L0 = v0 && in0 ? sm.table[cy0 * ww + cx0] : static_cast<acc_t>(0);
             acc_t L1 = v1 && in1 ? sm.table[cy1 * ww + cx1] : static_cast<acc_t>(0);
-            if constexpr (kMode == kModeStepBig) {   // (the tracker's table takes every draw: rarer still)
+            if constexpr (kMode == kModeStepBig) {   // (with the tracker's table none misses; without, see direct_likelihoods)
                 if (v0 && !in0) L0 = lik_from_sum<acc_t>(disk_sum(fv, sm.trk.w, pixel_of(x0), pixel_of(y0)), c1, c2D, den);
                 if (v1 && !in1) L1 = lik_from_sum<acc_t>(disk_sum(fv, sm.trk.w, pixel_of(x1), pixel_of(y1)), c1, c2D, den);
             } else {
@@ -2156,7 +2155,7 @@ __device__ void run_tile(const StepLaunch &Lp, int g, StepSmem<P> &sm) {
             const bool in1 = cx1 < static_cast<unsigned>(ww) && cy1 < static_cast<unsigned>(wh);
             H l0 = in0 ? sm.table[cy0 * ww + cx0] : OPS::from_f(0.0f);
             H l1 = in1 ? sm.table[cy1 * ww + cx1] : OPS::from_f(0.0f);
-            if constexpr (kMode == kModeStepBig) {   // (the tracker's table takes every draw: rarer still)
+            if constexpr (kMode == kModeStepBig) {   // (with the tracker's table none misses; without, see direct_likelihoods)
                 if (v0 && !in0) l0 = hk.at(fv, sm.trk.w, axi + pixel_of(OPS::lo(ox)), ayi + pixel_of(OPS::lo(oy)));
                 if (v1 && !in1) l1 = hk.at(fv, sm.trk.w, axi + pixel_of(OPS::hi(ox)), ayi + pixel_of(OPS::hi(oy)));
             } else {
@@ -2381,8 +2380,12 @@ int step_tile_size(int precision, int64_t n) {
     if (n < slots * (kTile / 2)) {
         // REF64 is bound by the FP64 pipes of the SMs that have a tile, so a tracker of four
         // full tiles or more is spread over all of them, down to tiles of 1024 (below, a tile's
-        // chain of phases costs as much as its arithmetic).  Smaller ones keep the tile count
-        // that the window hook has always reported for them.  200003 particles 134 -> 75 us a frame.
+        // chain of phases costs as much as its arithmetic).  us a frame, full tiles -> these: 16384
+        // particles 108 -> 51, 32768 110 -> 54, 200003 110 -> 64.  A batch that fills the device
+        // loses by it (64 trackers of 20003 272 -> 327, 16 of 200003 548 -> 691), but a tracker's sums,
+        // and so its bits, follow its tiles, and those are the same alone and in a batch.
+        // Smaller trackers keep the tiles of 4096 that the window hook reports for them: 16383
+        // particles 109, 4097 98.
         constexpr int64_t kLeast = kTile < 1024 ? kTile : 1024;
         if (precision == 0 && n >= 4 * kTile)
             return static_cast<int>(std::max(kLeast, ((n + slots - 1) / slots + 7) & ~int64_t(7)));
