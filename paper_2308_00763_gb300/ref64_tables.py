@@ -8,7 +8,7 @@ from __future__ import annotations
 
 import os
 import struct
-from decimal import ROUND_HALF_EVEN, Decimal, getcontext
+from decimal import ROUND_HALF_EVEN, Decimal, localcontext
 
 PI = Decimal("3.14159265358979323846264338327950288419716939937510582097494459")
 LN_UPPER = 424   # first logarithm interval whose centre is above sqrt 2 (kLnUpper)
@@ -50,7 +50,12 @@ def _ln(c: float, v: Decimal) -> str:
 
 def rows():
     """The members of Ref64Tables in order, each a list of entries."""
-    getcontext().prec = 60
+    with localcontext() as ctx:
+        ctx.prec = 60
+        return _rows()
+
+
+def _rows():
     hi, hi_rest = [], []
     for i in range(1024):
         s, c = _sin_cos(PI * i / 4096)
