@@ -24,10 +24,13 @@
 // a CTA's offspring take as long as the whole pool before them.  Every lane makes its eight tries
 // first, whatever the pool: over flat weights (the object lost) they decide every offspring, and a
 // warp's 64 for each were eight times the work.  Every offspring's tries and decision are those of
-// its own Philox stream either way.  Us a frame, 2048 a CTA without the list -> rejection_pool(N)
-// with it, on a tracked object: F16 2^20 161 -> 125, 200003 91 -> 51, F32 30001 119 -> 28, BF16 5003
-// 119 -> 19, REF64 20003 100 -> 44; over flat weights F16 2^20 54 -> 44, 150001 31 -> 20 (without
-// the lanes' own tries 70 and 51), sixteen trackers of 150001 133 -> 103 (487).
+// its own Philox stream either way.  A warp's lanes stay together: each iteration starts with a vote,
+// and a lane without tries to make sits it out (left to the loop's own branches, lanes that go on
+// with their offspring and lanes with a new one drift apart: REF64 2^20 677 us a frame against 507).
+// Us a frame, 2048 a CTA without the list -> rejection_pool(N) with it, on a tracked object: F16
+// 2^20 161 -> 126, 200003 91 -> 51, F32 30001 119 -> 28, BF16 5003 119 -> 19, REF64 20003 100 -> 44;
+// over flat weights F16 2^20 58 -> 47, 150001 32 -> 21 (without the lanes' own tries 74 and 54),
+// sixteen trackers of 150001 134 -> 96 (489).
 #include <math.h>
 
 #include "pf_ancestor.cuh"
@@ -67,7 +70,9 @@ __global__ void __launch_bounds__(kRejectionThreads) rejection_kernel(const Ance
 
     int e = static_cast<int>(threadIdx.x);   // the lane's offspring (pool index); >= pool: none
     int i = 0;                               // its next try (a multiple of 8)
-    while (e < pool) {
+    bool active = e < pool;                  // the lane makes tries (the warp's lanes stay together)
+    while (__any_sync(0xffffffffu, active)) {
+        if (!active) continue;
         const int jj = static_cast<int>(j0) + e;
         const uint32_t tag = 6u + (static_cast<uint32_t>(jj) << 8);
         // eight tries at a time: proposals (four Philox blocks) and gathers first, all eight
@@ -99,9 +104,10 @@ __global__ void __launch_bounds__(kRejectionThreads) rejection_kernel(const Ance
             T.anc[jj] = kd;
             e = static_cast<int>(atomicAdd(&s_next, 1u));
             i = 0;
+            active = e < pool;
         } else {
             i += 8;
-            if (*const_cast<volatile unsigned int *>(&s_next) >= static_cast<unsigned int>(pool)) break;
+            active = *const_cast<volatile unsigned int *>(&s_next) < static_cast<unsigned int>(pool);
         }
     }
     if (e < pool) {
