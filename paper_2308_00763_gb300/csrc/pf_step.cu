@@ -2261,8 +2261,9 @@ template <int P> struct MinBlocks {
     static constexpr int value = (P == 0 ? 512 : 1024) / kThreads > 0 ? (P == 0 ? 512 : 1024) / kThreads : 1;
 };
 
-// kWaves: the launch may have more tiles than CTAs.  (Without the loop over tiles the step mode holds
-// its registers better: F16 2^20 particles 19.66 -> 19.10 us a frame, F32 600001 17.1 -> 16.8.)
+// kWaves: the launch may have more tiles than CTAs.  (Without the loop over tiles the kernels hold
+// their registers better: F16 2^20 particles 19.66 -> 19.10 us a frame, F32 600001 17.1 -> 16.8,
+// multinomial F16 2^20 65.0 -> 63.9, 2^19 40.4 -> 39.8.)
 template <int P, int kMode, bool kWaves>
 __global__ void __launch_bounds__(kThreads, MinBlocks<P>::value) step_kernel(const StepLaunch Lp) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2340,7 +2341,8 @@ int configure_and_grid(int total_tiles) {
         return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
     };
     if (!allow(step_kernel<P, kModeStep, false>) || !allow(step_kernel<P, kModeStep, true>) ||
-        !allow(step_kernel<P, kModeStepBig, true>) || !allow(step_kernel<P, kModeCdf, true>) ||
+        !allow(step_kernel<P, kModeStepBig, true>) || !allow(step_kernel<P, kModeCdf, false>) ||
+        !allow(step_kernel<P, kModeCdf, true>) || !allow(step_kernel<P, kModePull, false>) ||
         !allow(step_kernel<P, kModePull, true>))
         return -1;
     int dev = 0, sms = 0, per_sm = 0;
@@ -2417,7 +2419,7 @@ int step_grid_size(int precision, int total_tiles) {
 // the stream is a step kernel (the previous frame), this launch is scheduled while that one
 // drains and waits for it on the device (griddepcontrol.wait) instead of the stream
 // serialising the two; captured into a CUDA graph as a programmatic dependency.
-template <int P, int kMode, bool kWaves>
+template <int P, int kMode>
 int launch_one(int grid, const StepLaunch &L, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
@@ -2429,20 +2431,23 @@ int launch_one(int grid, const StepLaunch &L, cudaStream_t s) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return static_cast<int>(cudaLaunchKernelEx(&cfg, step_kernel<P, kMode, kWaves>, L));
+    if constexpr (kMode != kModeStepBig) {
+        if (L.total_tiles <= grid) return static_cast<int>(cudaLaunchKernelEx(&cfg, step_kernel<P, kMode, false>, L));
+    }
+    return static_cast<int>(cudaLaunchKernelEx(&cfg, step_kernel<P, kMode, true>, L));
 }
 
-template <int kMode, bool kWaves = true>
+template <int kMode>
 int launch_mode(int precision, const StepLaunch &L, int grid, void *stream) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (L.total_tiles < 1) return 0;
     grid = std::max(1, std::min(grid, static_cast<int>(L.total_tiles)));   // (one wave: a CTA a tile)
     int rc = -1;
     switch (precision) {
-        case 0: rc = launch_one<0, kMode, kWaves>(grid, L, s); break;
-        case 1: rc = launch_one<1, kMode, kWaves>(grid, L, s); break;
-        case 2: rc = launch_one<2, kMode, kWaves>(grid, L, s); break;
-        case 3: rc = launch_one<3, kMode, kWaves>(grid, L, s); break;
+        case 0: rc = launch_one<0, kMode>(grid, L, s); break;
+        case 1: rc = launch_one<1, kMode>(grid, L, s); break;
+        case 2: rc = launch_one<2, kMode>(grid, L, s); break;
+        case 3: rc = launch_one<3, kMode>(grid, L, s); break;
         default: return -1;
     }
     if (rc != 0) return rc;
@@ -2453,7 +2458,6 @@ int launch_step(int precision, const StepLaunch &L, int grid, void *stream) {
     // a single tracker of at least two waves of tiles takes the instantiation with the
     // tracker table (the kernel checks the condition again per tile)
     if (L.ntrk == 1 && L.total_tiles >= 2 * grid) return launch_mode<kModeStepBig>(precision, L, grid, stream);
-    if (L.total_tiles <= std::max(1, grid)) return launch_mode<kModeStep, false>(precision, L, grid, stream);
     return launch_mode<kModeStep>(precision, L, grid, stream);
 }
 
